@@ -63,7 +63,7 @@ struct vg_workspace {
     DBuf<uint32_t> tord;                  // tile order buffer
     DBuf<short4> vbox;                    // voxel query: truncation boxes (2 per Gaussian)
     DBuf<float4> march_E;                 // ray march: o'.A_k per item
-    DBuf<float> tomo_dl;                  // fused tomography step: dL/dproj of one angle batch
+    DBuf<float> tomo_dl;                  // tomography backward: dL/dtau of one angle batch's pixels, padded rows
     uint32_t *tile_order = nullptr;       // longest-first tile order of the last bin_sort
     uint32_t *tile_order_bwd = nullptr;   // longest replay first, from the last forward (NULL: none)
     DBuf<uint32_t> treplay, tord_bwd;     // per-tile replay lengths and their order
@@ -94,6 +94,9 @@ namespace {
 constexpr int kDefaultPixelsFwd = 2;
 constexpr int kDefaultPixelsBwd = 1;
 constexpr int kDefaultChunk = 128;
+// Bytes of a view's weights that stay in an SM's L1 beside the other warps' data: up to there the backward's
+// item order does not matter (200 x 170 pixels, 136 KB: the sort's 45 us would be a third of the backward).
+constexpr long long kTomoL1Image = 160 * 1024;
 
 enum Stage { ST_PRE, ST_DEPTH, ST_SCAN, ST_DUP, ST_TILE, ST_RANGES, ST_FWD, ST_BWD, ST_CHAIN, ST_LOSS, ST_TFWD,
              ST_TBWD, ST_VOXEL, ST_MARCH, ST_COUNT };
@@ -1032,12 +1035,17 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
         }
         VG_TRY(ensure(ws, ws->views, vh.size(), "views"));
         VG_CUDA(ws, cudaMemcpyAsync(ws->views.p, vh.data(), vh.size() * sizeof(ViewInfo), cudaMemcpyHostToDevice, st));
+        // the backward's item order: by the tile of the footprint's centre (the last key: no footprint), once a
+        // view's weights no longer fit one SM's L1
+        const bool by_home = backward && (long long)beam->det_h * tomo_pitch(beam->det_w) * 4 > kTomoL1Image;
+        uint32_t *home = ws->skey[0].p, *order = nullptr;
         if (items > 0) {
             ProfScope ps(ws, ST_PRE, st);
             VG_CUDA(ws, cudaMemsetAsync(ws->depth.p, 0xFF, sizeof(uint32_t) * (size_t)items, st));
             VG_CUDA(ws, launch_tomo_preprocess(ws->g, ws->tomo_cs.p + 2 * (size_t)a0, nb, beam->det_w, beam->det_h,
                                                beam->pitch_u, beam->pitch_v, beam->u0, beam->v0, opts->tau_cut,
-                                               ws->rec.p, ws->count.p, ws->rect.p, ws->prect.p, st, &ws->launches));
+                                               ws->rec.p, ws->count.p, ws->rect.p, by_home ? home : nullptr, st,
+                                               &ws->launches));
         }
         {
             ProfScope ps(ws, ST_SCAN, st);
@@ -1069,24 +1077,25 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
         if (!proj_given) {
             ProfScope ps(ws, ST_TFWD, st);
             VG_CUDA(ws, launch_tomo_fwd(ws->ranges.p, n_tiles, tiles_x, (int)tpv, beam->det_w, beam->det_h,
-                                        ws->inst_item, ws->rec.p, ws->prect.p, proj_b, st, &ws->launches));
+                                        ws->inst_item, ws->rec.p, proj_b, st, &ws->launches));
         }
         const float *dl_b = dL_dproj ? dL_dproj + (size_t)a0 * det_px : nullptr;
-        if (fused) {   // the batch's share of the loss and its gradient dL/dproj
-            VG_TRY(ensure(ws, ws->tomo_dl, (size_t)nb * det_px, "loss gradient"));
+        if (backward) {   // the pixels' weights dL/dtau and, fused, the batch's share of the loss
+            VG_TRY(ensure(ws, ws->tomo_dl, (size_t)nb * beam->det_h * tomo_pitch(beam->det_w), "pixel weights"));
             ProfScope ps(ws, ST_LOSS, st);
-            VG_CUDA(ws, launch_l2_loss_acc(proj_b, target + (size_t)a0 * det_px, (long long)nb * det_px, scale, loss,
-                                           ws->tomo_dl.p, st, &ws->launches));
-            dl_b = ws->tomo_dl.p;
+            VG_CUDA(ws, launch_tomo_weights(proj_b, dl_b, fused ? target + (size_t)a0 * det_px : nullptr, scale, loss, nb,
+                                            beam->det_w, beam->det_h, ws->tomo_dl.p, st, &ws->launches));
         }
         if (backward && items > 0) {
             VG_TRY(ensure(ws, ws->grad, (size_t)items * 8, "gradient accumulators"));
             ws->grad_zero_n = 0;   // the tomography backward leaves its sums in the accumulator
-            VG_CUDA(ws, cudaMemsetAsync(ws->grad.p, 0, sizeof(float) * (size_t)items * 8, st));
             ProfScope ps(ws, ST_TBWD, st);
-            VG_CUDA(ws, launch_tomo_bwd(ws->ranges.p, n_tiles, tiles_x, (int)tpv, beam->det_w, beam->det_h,
-                                        ws->inst_item, ws->rec.p, ws->prect.p, proj_b, dl_b, ws->grad.p, st,
-                                        &ws->launches));
+            if (by_home)
+                VG_CUDA(ws, launch_radix_sort(home, nullptr, ws->skey[1].p, ws->sval[1].p, ws->skey[0].p, ws->sval[0].p, items,
+                                              nullptr, bits_for(n_tiles + 1), ws->hist.p, lookback_err_ptr(ws), &home, &order, st,
+                                              &ws->launches));
+            VG_CUDA(ws, launch_tomo_bwd(items, N, beam->det_w, beam->det_h, order, ws->count.p, ws->rec.p, ws->tomo_dl.p,
+                                        ws->grad.p, st, &ws->launches));
             VG_CUDA(ws, launch_tomo_chain(ws->g, ws->tomo_cs.p, A, (long long)a0 * N, items, beam->pitch_u,
                                           beam->pitch_v, beam->u0, beam->v0, ws->grad.p, dmu, dscale, dquat, dkappa,
                                           st, &ws->launches));

@@ -75,6 +75,41 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
+// Packed FP32 arithmetic (fma / add / mul.rn.f32x2): two independent IEEE operations, each rounded
+// exactly as its scalar counterpart, in one issue slot.  The pair and blend loops are bound by
+// issue slots (70-85% of cycles issue while the FMA pipe is active on 35-45% of them), so halving
+// the instructions of the same operations is what they gain from.
+struct F2 {
+    unsigned long long v;   // low half: first value
+};
+__device__ __forceinline__ F2 f2_pack(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ F2 f2_dup(float a) { return f2_pack(a, a); }
+__device__ __forceinline__ void f2_unpack(F2 p, float &a, float &b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(p.v)); }
+__device__ __forceinline__ float f2_sum(F2 p) {
+    float a, b;
+    f2_unpack(p, a, b);
+    return a + b;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
 // Programmatic dependent launch: every kernel of the library is launched with programmatic
 // stream serialisation, so the next kernel's CTAs are scheduled while the previous kernel's
 // last wave drains.  pdl_entry() must run first in every kernel: it blocks until the previous
@@ -123,7 +158,7 @@ cudaError_t launch_preprocess(const GaussIn &g, const ViewInfo *views_d, int n_v
 
 cudaError_t launch_tomo_preprocess(const GaussIn &g, const float *cs_d /* [A][2] cos, sin */, int n_angles,
                                    int det_w, int det_h, float pitch_u, float pitch_v, float u0, float v0,
-                                   float tau_cut, float4 *rec, uint32_t *count, short4 *rect, short4 *prect,
+                                   float tau_cut, float4 *rec, uint32_t *count, short4 *rect, uint32_t *home,
                                    cudaStream_t st, long long *launches);
 
 // Error bits latched in the workspace's device flag word.
@@ -223,12 +258,21 @@ cudaError_t launch_chain(const GaussIn &g, const ViewInfo *views_d, int n_views,
                          long long *launches);
 
 cudaError_t launch_tomo_fwd(const uint2 *ranges, long long n_tiles, int tiles_x, int tiles_per_view, int det_w,
-                            int det_h, const uint32_t *sorted_item, const float4 *rec, const short4 *prect,
-                            float *proj, cudaStream_t st, long long *launches);
+                            int det_h, const uint32_t *sorted_item, const float4 *rec, float *proj, cudaStream_t st,
+                            long long *launches);
 
-cudaError_t launch_tomo_bwd(const uint2 *ranges, long long n_tiles, int tiles_x, int tiles_per_view, int det_w,
-                            int det_h, const uint32_t *sorted_item, const float4 *rec, const short4 *prect,
-                            const float *proj, const float *dL_dproj, float *grad_acc, cudaStream_t st,
+// The pixel weights of the tomography backward, dL/dtau = -proj dL/dproj, as rows of
+// tomo_pitch(det_w) floats (32-byte aligned, padding zero): from dL, or (dL NULL) from the L2 loss
+// scale sum (proj - target)^2, which is then added to *loss.
+inline int tomo_pitch(int det_w) { return (det_w + 7) & ~7; }
+cudaError_t launch_tomo_weights(const float *proj, const float *dL, const float *target, float scale, float *loss,
+                                int n_views, int det_w, int det_h, float *weights, cudaStream_t st,
+                                long long *launches);
+
+// Writes the 8 sums of every item (zeros for one without a footprint) into acc, the items taken in
+// the given order (NULL: their own).
+cudaError_t launch_tomo_bwd(long long n_items, int n_per_view, int det_w, int det_h, const uint32_t *order,
+                            const uint32_t *count, const float4 *rec, const float *weights, float *acc, cudaStream_t st,
                             long long *launches);
 
 cudaError_t launch_tomo_chain(const GaussIn &g, const float *cs_d, int n_angles, long long item0, long long n_items,
@@ -237,8 +281,5 @@ cudaError_t launch_tomo_chain(const GaussIn &g, const float *cs_d, int n_angles,
 
 cudaError_t launch_l2_loss(const float *x, const float *y, long long n, float scale, float *loss, float *grad,
                            cudaStream_t st, long long *launches);
-// The same without zeroing *loss first (accumulates across calls).
-cudaError_t launch_l2_loss_acc(const float *x, const float *y, long long n, float scale, float *loss, float *grad,
-                               cudaStream_t st, long long *launches);
 
 }  // namespace vg
