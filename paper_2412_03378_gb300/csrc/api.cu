@@ -63,6 +63,7 @@ struct vg_workspace {
     DBuf<uint32_t> tord;                  // tile order buffer
     DBuf<short4> vbox;                    // voxel query: truncation boxes (2 per Gaussian)
     DBuf<float4> march_E;                 // ray march: o'.A_k per item
+    DBuf<float4> march_part;              // ray march: colour and transmittance per (group of passes, pixel)
     DBuf<float> tomo_dl;                  // tomography backward: dL/dtau of one angle batch's pixels, padded rows
     uint32_t *tile_order = nullptr;       // longest-first tile order of the last bin_sort
     uint32_t *tile_order_bwd = nullptr;   // longest replay first, from the last forward (NULL: none)
@@ -97,6 +98,7 @@ constexpr int kDefaultChunk = 128;
 // Bytes of a view's weights that stay in an SM's L1 beside the other warps' data: up to there the backward's
 // item order does not matter (200 x 170 pixels, 136 KB: the sort's 45 us would be a third of the backward).
 constexpr long long kTomoL1Image = 160 * 1024;
+constexpr long long kMarchCtas = 4096;   // ray march: CTAs wanted (27 per SM)
 
 enum Stage { ST_PRE, ST_DEPTH, ST_SCAN, ST_DUP, ST_TILE, ST_RANGES, ST_FWD, ST_BWD, ST_CHAIN, ST_LOSS, ST_TFWD,
              ST_TBWD, ST_VOXEL, ST_MARCH, ST_COUNT };
@@ -285,6 +287,7 @@ vg_status vg_workspace_destroy(vg_workspace *ws) {
     release(ws->tord_bwd);
     release(ws->vbox);
     release(ws->march_E);
+    release(ws->march_part);
     release(ws->tomo_dl);
     if (ws->h_total) cudaFreeHost(ws->h_total);
     for (auto &r : ws->prof) {
@@ -763,11 +766,27 @@ vg_status vg_ray_march(vg_workspace *ws, float t_near, float t_far, int32_t n_sa
     if (err_map && !raster_rgb) return fail(ws, VG_ERR_INVALID_ARG, "err_map needs raster_rgb");
     cudaStream_t st = (cudaStream_t)stream;
     VG_TRY(ensure(ws, ws->march_E, (size_t)ws->n_items, "ray-march scratch"));
+    // Groups of passes per tile: enough CTAs to spread the longest lists (kMarchCtas in all), one when the image has
+    // them by itself or when an early stop makes a pass depend on the ones before.  The partial results' buffer is
+    // sized by the views alone; where it may not grow (fixed capacity, a capturing stream), what it holds decides.
+    int groups = 1;
+    if (ws->opts.T_stop == 0.0f && ws->n_tiles > 0 && ws->n_pixels > 0) {
+        const long long px = ws->n_pixels;
+        groups = (int)std::min<long long>(64, (kMarchCtas + ws->n_tiles - 1) / ws->n_tiles);
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        VG_CUDA(ws, cudaStreamIsCapturing(st, &cap));
+        const bool keep = cap != cudaStreamCaptureStatusNone || (ws->march_part.p && (ws->opts.flags & VG_FLAG_FIXED_CAPACITY));
+        if (keep)
+            groups = (int)std::min<long long>(groups, (long long)ws->march_part.n / px);
+        else if (groups > 1)
+            VG_TRY(ensure(ws, ws->march_part, (size_t)(groups * px), "ray-march partial results"));
+        groups = std::max(groups, 1);
+    }
     ProfScope ps(ws, ST_MARCH, st);
-    VG_CUDA(ws, launch_ray_march(ws->g, ws->views.p, ws->tile_view.p, ws->n_tiles, ws->bp.tile_px, ws->n_items,
-                                 ws->ranges.p,
-                                 ws->inst_item, ws->rec.p, ws->count.p, ws->prect.p, ws->march_E.p, t_near, t_far,
-                                 n_samples, ws->opts.T_stop, ws->opts.bg, raster_rgb, rgb, T, err_map, st,
+    VG_CUDA(ws, launch_ray_march(ws->g, ws->views.p, ws->tile_view.p, (const int *)ws->tile_order, ws->n_tiles,
+                                 ws->bp.tile_px, ws->n_items, ws->n_pixels, ws->ranges.p, ws->inst_item, ws->rec.p,
+                                 ws->count.p, ws->prect.p, ws->march_E.p, t_near, t_far, n_samples, ws->opts.T_stop,
+                                 groups, ws->march_part.p, ws->opts.bg, raster_rgb, rgb, T, err_map, st,
                                  &ws->launches));
     return VG_OK;
 }

@@ -241,15 +241,17 @@ cudaError_t launch_voxel_dup(const uint32_t *offsets, const short4 *box, const V
 cudaError_t launch_voxel_eval(const uint2 *ranges, const uint32_t *sorted, const float4 *rec, const short4 *box,
                               const VoxelGrid &grid, float *out, cudaStream_t st, long long *launches);
 
-// Ray-marching reference (march.cu): one CTA of tile_px threads per tile (one pixel each); E
-// receives (o'.A0, o'.A1, o'.A2) per item (scratch);
-// rgb / T_out / err (max over channels of |rgb - raster|) are each optional.
-cudaError_t launch_ray_march(const GaussIn &g, const ViewInfo *views_d, const int *tile_view, long long n_tiles,
-                             int tile_px,
-                             long long n_items, const uint2 *ranges, const uint32_t *sorted_item, const float4 *rec,
+// Ray-marching reference (march.cu): CTAs of tile_px threads (one pixel each), `groups` of them per
+// tile over consecutive samples; E receives (o'.A0, o'.A1, o'.A2, range of t) per item (scratch);
+// rgb / T_out / err (max over channels of |rgb - raster|) are each optional.  groups > 1 needs
+// T_stop = 0 and part of groups x n_pixels.
+cudaError_t launch_ray_march(const GaussIn &g, const ViewInfo *views_d, const int *tile_view, const int *tile_order,
+                             long long n_tiles, int tile_px, long long n_items, long long n_pixels,
+                             const uint2 *ranges, const uint32_t *sorted_item, const float4 *rec,
                              const uint32_t *count, const short4 *prect, float4 *E, float t_near, float t_far,
-                             int n_samples, float T_stop, const float bg[3], const float *raster, float *rgb,
-                             float *T_out, float *err, cudaStream_t st, long long *launches);
+                             int n_samples, float T_stop, int groups, float4 *part, const float bg[3],
+                             const float *raster, float *rgb, float *T_out, float *err, cudaStream_t st,
+                             long long *launches);
 
 // The chain reads grad_acc and leaves every item it reads zero again (an all-zero row is left
 // as it is), so a following backward needs no clearing pass.
