@@ -93,6 +93,10 @@ namespace {
 // Measured on the 1M-Gaussian 1280x832 workload (GB300, footprint culling on): forward
 // 0.53 / 0.49 / 0.74 ms and backward 1.32 / 1.16 / 1.19 ms for 1 / 2 / 4 pixels per thread.
 constexpr int kDefaultPixelsFwd = 2;
+// Up to this many tiles (16 per SM) the forward takes one pixel per thread: more warps per tile, each with fewer
+// records to visit, and several records evaluated at once.  One / two pixels per thread: 64 tiles 42 / 73 us, 672 tiles
+// 72 / 110 us, 1,040 tiles 93 / 126 us, 1,900 tiles 140 / 178 us, 4,160 tiles 156 / 128 us.
+constexpr long long kOnePixelTiles = 152 * 16;
 constexpr int kDefaultPixelsBwd = 1;
 constexpr int kDefaultChunk = 128;
 // Bytes of a view's weights that stay in an SM's L1 beside the other warps' data: up to there the backward's
@@ -483,7 +487,7 @@ static vg_status preprocess_impl(vg_workspace *ws, const vg_gaussians *g, const 
     ws->n_pixels = pix_base;
     ws->bp.tau_skip = opts->alpha_min > 0.0f ? (float)(-std::log1p(-(double)opts->alpha_min)) : 0.0f;
     ws->bp.tau_max = opts->tau_max;
-    ws->ppt_fwd = opts->pixels_per_thread ? opts->pixels_per_thread : (ws->tuned_fwd ? ws->tuned_fwd : kDefaultPixelsFwd);
+    ws->ppt_fwd = opts->pixels_per_thread ? opts->pixels_per_thread : (ws->tuned_fwd ? ws->tuned_fwd : (tile_base <= kOnePixelTiles ? 1 : kDefaultPixelsFwd));
     ws->ppt_bwd = opts->pixels_per_thread ? opts->pixels_per_thread : (ws->tuned_bwd ? ws->tuned_bwd : kDefaultPixelsBwd);
     ws->bp.chunk_fwd = opts->chunk ? opts->chunk : (ws->tuned_chunk_fwd ? ws->tuned_chunk_fwd : kDefaultChunk);
     ws->bp.chunk_bwd = opts->chunk ? opts->chunk : (ws->tuned_chunk_bwd ? ws->tuned_chunk_bwd : kDefaultChunk);

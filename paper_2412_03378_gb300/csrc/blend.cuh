@@ -26,21 +26,61 @@ __device__ __forceinline__ PixelRay pixel_ray(const ViewInfo &V, int x, int y) {
     return p;
 }
 
-// Record layout (6 x float4):
-//   r0 = (A0.x, A0.y, A0.z, A1.x)  r1 = (A1.y, A1.z, A2.x, A2.y)  r2 = (A2.z, C0.x, C0.y, C0.z)
-//   r3 = (C1.x, C1.y, C1.z, C2.x)  r4 = (C2.y, C2.z, px0, py0)     r5 = (log2(kappa sqrt(2pi)), r, g, b)
+// Record layout (6 x float4): (A0, C0), (A1, C1), (A2, C2) component by component, then the rest,
+//   q0 = (A0.x, C0.x, A0.y, C0.y)  q1 = (A0.z, C0.z, A1.x, C1.x)  q2 = (A1.y, C1.y, A1.z, C1.z)
+//   q3 = (A2.x, C2.x, A2.y, C2.y)  q4 = (A2.z, C2.z, px0, py0)    q5 = (log2(kappa sqrt(2pi)), r, g, b)
 // d' = A0 dx + A1 dy + A2, o' x d' = C0 dx + C1 dy + C2 with (dx, dy) = pixel - (px0, py0);
 //   tau = kappa sqrt(2 pi) |d_c| / |d'| exp(-|o' x d'|^2 / (2 |d'|^2))   (Eq. 19, unit-ray form).
+// Both vectors are formed by the same operations on the same (dx, dy), so each component of d' is
+// computed together with that of o' x d' in one packed operation, and so are |d'|^2 and
+// |o' x d'|^2; the record's pairs come out of its 16-byte loads as the packed operands.
 // Every pixel is evaluated by the same operations, whatever the pixel layout of the kernel:
 //   dx = x - px0, dy = y - py0 (rounded), d'_c = fma(A1_c, dy, fma(A0_c, dx, A2_c)) and the same
 //   for o' x d' with C.
 // The inner term depends on the pixel column only, so the pixels of a thread that share a column
 // share it (ColBase), and forward and backward compute identical bits for a pixel -- and take
 // identical skip and clamp decisions -- with any pixels-per-thread setting of either kernel.
-struct PairEval {
-    float dx, dy;
-    float dp[3], cr[3];
-    float rs, m2, tau;
+struct RecPairs {
+    F2 ac0[3], ac1[3], ac2[3];   // (A_k, C_k) component by component
+    float px0, py0;
+    float4 q5;
+};
+
+__device__ __forceinline__ void load_rec(const float4 *rec, RecPairs &r) {   // 16-byte aligned, shared memory
+    const ulonglong2 *u = reinterpret_cast<const ulonglong2 *>(rec);
+    const ulonglong2 u0 = u[0], u1 = u[1], u2 = u[2], u3 = u[3];
+    const float4 q4 = rec[4];
+    r.ac0[0].v = u0.x, r.ac0[1].v = u0.y, r.ac0[2].v = u1.x;
+    r.ac1[0].v = u1.y, r.ac1[1].v = u2.x, r.ac1[2].v = u2.y;
+    r.ac2[0].v = u3.x, r.ac2[1].v = u3.y, r.ac2[2] = f2_pack(q4.x, q4.y);
+    r.px0 = q4.z, r.py0 = q4.w;
+    r.q5 = rec[5];
+}
+
+// Splat mode needs the first two rows of C alone (A = (0, 0, e_z)): its records are 3 x float4,
+//   q0 = (C0.x, C0.y, C1.x, C1.y)  q1 = (C2.x, C2.y, px0, py0)  q2 = (log2 o, r, g, b).
+struct SplatRec {
+    float c0[2], c1[2], c2[2];
+    float px0, py0;
+    float4 q5;
+};
+
+__device__ __forceinline__ void load_rec(const float4 *rec, SplatRec &r) {
+    const float4 q0 = rec[0], q1 = rec[1];
+    r.c0[0] = q0.x, r.c0[1] = q0.y, r.c1[0] = q0.z, r.c1[1] = q0.w, r.c2[0] = q1.x, r.c2[1] = q1.y;
+    r.px0 = q1.z, r.py0 = q1.w;
+    r.q5 = rec[2];
+}
+
+template <bool SPLAT>
+struct RecOf {   // the record as the blend kernels hold it, and its float4s in memory
+    using type = RecPairs;
+    static constexpr int kF4 = kRecF4;
+};
+template <>
+struct RecOf<true> {
+    using type = SplatRec;
+    static constexpr int kF4 = 3;
 };
 
 // A thread owns P pixels of a tile of tw x th pixels (16 x 16, 32 x 16 or 16 x 8; P = 1, 2 or 4);
@@ -56,7 +96,7 @@ template <int P>
 struct PixLayout {
     static constexpr int kBoxW = P == 4 ? 16 : 8;
     // register caps that keep the occupancy of 16 x 16 tiles (forward / backward)
-    static constexpr int kFwdRegs = P == 2 ? 73 : 85;
+    static constexpr int kFwdRegs = P == 2 ? 73 : (P == 1 ? 80 : 85);
     static constexpr int kBwdRegs = P == 1 ? 56 : (P == 2 ? 96 : 128);
     __device__ static void origin(int t, int tw, int &x, int &y) {
         const int w = t >> 5, l = t & 31;
@@ -75,6 +115,13 @@ struct PixLayout {
     __host__ __device__ static constexpr int ox(int k) { return P == 4 ? (k & 1) : 0; }
     __host__ __device__ static constexpr int oy(int k) { return P == 4 ? (k >> 1) : (P == 2 ? k : 0); }
 };
+
+// With few tiles the longest list's CTA decides a blend kernel's time while other SMs idle: two CTAs then
+// share a tile's warps (each stages the list itself), up to 8 tiles per SM.  Forward / backward at one pixel
+// per thread with 1 and 2 CTAs per tile: 64 tiles (2,000 Gaussians, no early stop) 54.7 -> 42.3 us / -, 1,040
+// tiles (100,000 Gaussians) 97.3 -> 92.6 / 156.7 -> 149.8 us, 672 tiles (splat mode) 86.8 -> 77.9 / 190.9 -> 179.7 us;
+// 1,900 tiles 139.5 -> 140.9 us, 4,160 tiles 267 -> 275 us; 4 CTAs per tile 44.4, 108.5, 83.5 us.
+inline int tile_split(long long n_tiles, int threads) { return n_tiles <= 152 * 8 && threads >= 64 ? 2 : 1; }
 
 // Bounds of the pixels a warp owns, for the warp-uniform footprint test of each record.
 struct WarpBox {
@@ -106,7 +153,7 @@ __device__ __forceinline__ bool box_inside(const WarpBox &b, const short4 &r) {
 }
 
 __device__ __forceinline__ bool pixel_outside(int x, int y, const short4 &r) {
-    return x < r.x || x > r.z || y < r.y || y > r.w;
+    return (x < r.x) | (x > r.z) | (y < r.y) | (y > r.w);   // no branches: the caller's evaluation stays in line
 }
 
 // Conservative opacity test of one record against a warp's pixel box, for blending with
@@ -151,18 +198,32 @@ __device__ __forceinline__ float quad_edge_min(float h, float rh, float hc, floa
     return fmaf(fmaf(h, s, 2.0f * hc), s, c0);
 }
 
-// Per record, the Gram matrices the test needs: G = A^T A and K = C^T C over the columns
-// (A0, A1, A2), (C0, C1, C2), packed as (g00 g01 g02 g11) (g12 g22 k00 k01) (k02 k11 k12 k22).
-constexpr int kCullF4 = 3;
+// What the test needs of a record, in shared memory arrays of kCullF4 float4 (by row or by record) and
+// (px0, py0, log2 K, |A0|), |A1|: the Gram matrices G = A^T A and K = C^T C over the columns (A0, A1,
+// A2), (C0, C1, C2), packed as (g00 g01 g02 g11) (g12 g22 k00 k01) (k02 k11 k12 k22); in splat mode
+// (k00 k01 k02 k11) (k12 k22 - -).
+template <bool SPLAT>
+constexpr int kCullF4 = SPLAT ? 2 : 3;
 
-__device__ __forceinline__ void cull_row(const float4 &r0, const float4 &r1, const float4 &r2, const float4 &r3,
-                                         const float4 &r4, float4 out[kCullF4]) {
-    const float A0[3] = {r0.x, r0.y, r0.z}, A1[3] = {r0.w, r1.x, r1.y}, A2[3] = {r1.z, r1.w, r2.x};
-    const float C0[3] = {r2.y, r2.z, r2.w}, C1[3] = {r3.x, r3.y, r3.z}, C2[3] = {r3.w, r4.x, r4.y};
-    auto dot = [](const float *a, const float *b) { return fmaf(a[0], b[0], fmaf(a[1], b[1], a[2] * b[2])); };
-    out[0] = make_float4(dot(A0, A0), dot(A0, A1), dot(A0, A2), dot(A1, A1));
-    out[1] = make_float4(dot(A1, A2), dot(A2, A2), dot(C0, C0), dot(C0, C1));
-    out[2] = make_float4(dot(C0, C2), dot(C1, C1), dot(C1, C2), dot(C2, C2));
+template <bool SPLAT>
+__device__ __forceinline__ void cull_row(const float4 *q, float4 *out, float4 &ref, float &a1) {
+    if constexpr (SPLAT) {
+        const float C0[2] = {q[0].x, q[0].y}, C1[2] = {q[0].z, q[0].w}, C2[2] = {q[1].x, q[1].y};
+        auto dot = [](const float *a, const float *b) { return fmaf(a[0], b[0], a[1] * b[1]); };
+        out[0] = make_float4(dot(C0, C0), dot(C0, C1), dot(C0, C2), dot(C1, C1));
+        out[1] = make_float4(dot(C1, C2), dot(C2, C2), 0.0f, 0.0f);
+        ref = make_float4(q[1].z, q[1].w, q[2].x, 0.0f);
+        a1 = 0.0f;
+    } else {
+        const float A0[3] = {q[0].x, q[0].z, q[1].x}, A1[3] = {q[1].z, q[2].x, q[2].z}, A2[3] = {q[3].x, q[3].z, q[4].x};
+        const float C0[3] = {q[0].y, q[0].w, q[1].y}, C1[3] = {q[1].w, q[2].y, q[2].w}, C2[3] = {q[3].y, q[3].w, q[4].y};
+        auto dot = [](const float *a, const float *b) { return fmaf(a[0], b[0], fmaf(a[1], b[1], a[2] * b[2])); };
+        out[0] = make_float4(dot(A0, A0), dot(A0, A1), dot(A0, A2), dot(A1, A1));
+        out[1] = make_float4(dot(A1, A2), dot(A2, A2), dot(C0, C0), dot(C0, C1));
+        out[2] = make_float4(dot(C0, C2), dot(C1, C1), dot(C1, C2), dot(C2, C2));
+        ref = make_float4(q[4].z, q[4].w, q[5].x, sqrtf(out[0].x));
+        a1 = sqrtf(out[0].w);
+    }
 }
 
 // The test of the record (px0, py0, log2 K from the record; Gram matrices from cull_row; sg00 =
@@ -199,37 +260,51 @@ __device__ __forceinline__ bool box_may_blend(const float4 &ga, const float4 &gb
 }
 
 struct ColBase {
-    float dx;              // x - px0 of the column
-    float ip[3], ic[3];    // fma(A0, dx, A2) and fma(C0, dx, C2)
+    float dx;    // x - px0 of the column
+    F2 i[3];     // fma(A0, dx, A2) and fma(C0, dx, C2)
 };
 
-__device__ __forceinline__ void col_base(const float4 &r0, const float4 &r1, const float4 &r2, const float4 &r3,
-                                         const float4 &r4, float x, ColBase &b) {
-    b.dx = __fsub_rn(x, r4.z);
-    b.ip[0] = fmaf(r0.x, b.dx, r1.z);
-    b.ip[1] = fmaf(r0.y, b.dx, r1.w);
-    b.ip[2] = fmaf(r0.z, b.dx, r2.x);
-    b.ic[0] = fmaf(r2.y, b.dx, r3.w);
-    b.ic[1] = fmaf(r2.z, b.dx, r4.x);
-    b.ic[2] = fmaf(r2.w, b.dx, r4.y);
+__device__ __forceinline__ void col_base(const RecPairs &r, float x, ColBase &b) {
+    b.dx = __fsub_rn(x, r.px0);
+    const F2 dx = f2_dup(b.dx);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) b.i[k] = f2_fma(r.ac0[k], dx, r.ac2[k]);
 }
 
-// d', o' x d', (dx, dy) and tau (unclamped) of the pixel in row y of the column b.
-__device__ __forceinline__ void pair_eval_col(const float4 &r0, const float4 &r1, const float4 &r3, const float4 &r4,
-                                              const float4 &r5, const ColBase &b, float y, float Lp, PairEval &e) {
-    e.dx = b.dx;
-    e.dy = __fsub_rn(y, r4.w);
-    e.dp[0] = fmaf(r0.w, e.dy, b.ip[0]);
-    e.dp[1] = fmaf(r1.x, e.dy, b.ip[1]);
-    e.dp[2] = fmaf(r1.y, e.dy, b.ip[2]);
-    e.cr[0] = fmaf(r3.x, e.dy, b.ic[0]);
-    e.cr[1] = fmaf(r3.y, e.dy, b.ic[1]);
-    e.cr[2] = fmaf(r3.z, e.dy, b.ic[2]);
-    const float a = fmaf(e.dp[0], e.dp[0], fmaf(e.dp[1], e.dp[1], __fmul_rn(e.dp[2], e.dp[2])));
-    const float q = fmaf(e.cr[0], e.cr[0], fmaf(e.cr[1], e.cr[1], __fmul_rn(e.cr[2], e.cr[2])));
+// (|d'|^2, |o' x d'|^2) of the pixel at dy in the column b.
+__device__ __forceinline__ F2 pair_squares(const RecPairs &r, const ColBase &b, float dy) {
+    const F2 d = f2_dup(dy);
+    const F2 t0 = f2_fma(r.ac1[0], d, b.i[0]), t1 = f2_fma(r.ac1[1], d, b.i[1]), t2 = f2_fma(r.ac1[2], d, b.i[2]);
+    return f2_fma(t0, t0, f2_fma(t1, t1, f2_mul(t2, t2)));
+}
+
+// dy, 1 / |d'|, m^2 and tau (unclamped) of the pixel in row y of the column b.
+struct PairEval {
+    float dy, rs, m2, tau;
+};
+
+__device__ __forceinline__ void pair_eval_col(const RecPairs &r, const ColBase &b, float y, float Lp, PairEval &e) {
+    e.dy = __fsub_rn(y, r.py0);
+    float a, q;
+    f2_unpack(pair_squares(r, b, e.dy), a, q);
     e.rs = rsqrt_approx(a);
     e.m2 = __fmul_rn(q, __fmul_rn(e.rs, e.rs));
-    e.tau = __fmul_rn(ex2_approx(fmaf(e.m2, -kHalfLog2e, __fadd_rn(r5.x, Lp))), e.rs);
+    e.tau = __fmul_rn(ex2_approx(fmaf(e.m2, -kHalfLog2e, __fadd_rn(r.q5.x, Lp))), e.rs);
+}
+
+// tau of the two pixels in rows y of the column b: the operations of pair_eval_col, packed over the
+// rows where both halves come from one register pair.
+__device__ __forceinline__ void pair_tau2(const RecPairs &r, const ColBase &b, const F2 &y, const F2 &Lp, float tau[2]) {
+    float dy[2], a[2], q[2], w[2];
+    f2_unpack(f2_add(y, f2_dup(-r.py0)), dy[0], dy[1]);
+    f2_unpack(pair_squares(r, b, dy[0]), a[0], q[0]);
+    f2_unpack(pair_squares(r, b, dy[1]), a[1], q[1]);
+    const F2 rs = f2_pack(rsqrt_approx(a[0]), rsqrt_approx(a[1]));
+    f2_unpack(f2_mul(rs, rs), w[0], w[1]);
+    const F2 m2 = f2_pack(__fmul_rn(q[0], w[0]), __fmul_rn(q[1], w[1]));
+    float e[2];
+    f2_unpack(f2_fma(m2, f2_dup(-kHalfLog2e), f2_add(f2_dup(r.q5.x), Lp)), e[0], e[1]);
+    f2_unpack(f2_mul(f2_pack(ex2_approx(e[0]), ex2_approx(e[1])), rs), tau[0], tau[1]);
 }
 
 // ------------------------------------------------------------------ splat mode (Eq. 5-7)
@@ -244,21 +319,20 @@ struct SplatCol {
     float i0, i1;    // fma(C0, dx, C2), two components
 };
 
-__device__ __forceinline__ void splat_col(const float4 &r2, const float4 &r3, const float4 &r4, float x, SplatCol &b) {
-    b.dx = __fsub_rn(x, r4.z);
-    b.i0 = fmaf(r2.y, b.dx, r3.w);
-    b.i1 = fmaf(r2.z, b.dx, r4.x);
+__device__ __forceinline__ void splat_col(const SplatRec &r, float x, SplatCol &b) {
+    b.dx = __fsub_rn(x, r.px0);
+    b.i0 = fmaf(r.c0[0], b.dx, r.c2[0]);
+    b.i1 = fmaf(r.c0[1], b.dx, r.c2[1]);
 }
 
 // (dx, dy) and q = |C u|^2 of the pixel in row y of the column b (the same operations for every
 // pixel layout); returns the unclamped opacity o G'(p).
-__device__ __forceinline__ float splat_at(const float4 &r3, const float4 &r4, const float4 &r5, const SplatCol &b,
-                                          float y, float &dx, float &dy, float &q) {
+__device__ __forceinline__ float splat_at(const SplatRec &r, const SplatCol &b, float y, float &dx, float &dy, float &q) {
     dx = b.dx;
-    dy = __fsub_rn(y, r4.w);
-    const float c0 = fmaf(r3.x, dy, b.i0), c1 = fmaf(r3.y, dy, b.i1);
+    dy = __fsub_rn(y, r.py0);
+    const float c0 = fmaf(r.c1[0], dy, b.i0), c1 = fmaf(r.c1[1], dy, b.i1);
     q = fmaf(c0, c0, __fmul_rn(c1, c1));
-    return ex2_approx(fmaf(q, -kHalfLog2e, r5.x));
+    return ex2_approx(fmaf(q, -kHalfLog2e, r.q5.x));
 }
 
 // The opacity box test of the splat mode: box_may_blend with the record's A = (0, 0, e_z)
@@ -272,6 +346,18 @@ __device__ __forceinline__ BoxCull box_cull_splat(const WarpBox &b, float alpha_
     c.l2dmax = 1e-4f;
     c.l2tskip = __log2f(alpha_min);
     return c;
+}
+
+// The opacity test of a staged record: `row(k)` its kCullF4 float4.
+template <bool SPLAT, typename Row>
+__device__ __forceinline__ bool rec_may_blend(Row row, const float4 &ref, float a1, const BoxCull &bc) {
+    if constexpr (SPLAT) {
+        const float4 k0 = row(0), k1 = row(1);
+        return box_may_blend(make_float4(0.0f, 0.0f, 0.0f, 0.0f), make_float4(0.0f, 1.0f, k0.x, k0.y),
+                             make_float4(k0.z, k0.w, k1.x, k1.y), ref.x, ref.y, ref.z, 0.0f, 0.0f, bc);
+    } else {
+        return box_may_blend(row(0), row(1), row(2), ref.x, ref.y, ref.z, ref.w, a1, bc);
+    }
 }
 
 // Asynchronous global-to-shared copies (cp.async): 16 bytes (both addresses 16-byte aligned)

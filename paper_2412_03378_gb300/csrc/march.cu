@@ -147,16 +147,14 @@ k_ray_march(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vie
                     m &= m - 1;
                     if (!live || pixel_outside(x, y, srect[j])) continue;
                     const float4 *rr = &srec[j * (kRecF4 + 1)];
-                    const float4 r0 = rr[0], r1 = rr[1], r2 = rr[2], r3 = rr[3], r4 = rr[4], r5 = rr[5], e4 = rr[6];
-                    const float dx = xf - r4.z, dy = yf - r4.w;
-                    const float d0 = fmaf(r0.x, dx, fmaf(r0.w, dy, r1.z));
-                    const float d1 = fmaf(r0.y, dx, fmaf(r1.x, dy, r1.w));
-                    const float d2 = fmaf(r0.z, dx, fmaf(r1.y, dy, r2.x));
-                    const float q0 = fmaf(r2.y, dx, fmaf(r3.x, dy, r3.w));
-                    const float q1 = fmaf(r2.z, dx, fmaf(r3.y, dy, r4.x));
-                    const float q2 = fmaf(r2.w, dx, fmaf(r3.z, dy, r4.y));
-                    const float a = fmaf(d0, d0, fmaf(d1, d1, d2 * d2));
-                    const float qq = fmaf(q0, q0, fmaf(q1, q1, q2 * q2));
+                    RecPairs R;
+                    load_rec(rr, R);
+                    const float4 r5 = R.q5, e4 = rr[6];
+                    ColBase col;
+                    col_base(R, xf, col);
+                    const float dx = col.dx, dy = yf - R.py0;
+                    float a, qq;
+                    f2_unpack(pair_squares(R, col, dy), a, qq);
                     const float bq = fmaf(e4.x, dx, fmaf(e4.y, dy, e4.z));
                     const float ia = 1.0f / a;
                     const float lp = fmaf(-qq * ia, kHalfLog2e, r5.x - kLog2Sqrt2Pi);   // log2(kappa exp(-m^2/2))

@@ -57,7 +57,7 @@ k_preprocess(GaussIn g, const ViewInfo *__restrict__ views, int n_views, float z
             if (state == 2) {
                 cnt = (uint32_t)(rc.z - rc.x + 1) * (uint32_t)(rc.w - rc.y + 1);
                 float dir[3], len, rgb[3] = {0.0f, 0.0f, 0.0f}, raw[3];
-                float rrow[4 * kRecF4];
+                float rrow[4 * kRecF4];   // A (9), C (9), px0, py0, log2 K, colour: paired up as they are stored
                 view_dir(V, mu, dir, len);
                 if (SH3)
                     eval_colour_sh3(reinterpret_cast<const float4 *>(row), dir, rgb, raw, g.softplus_beta);
@@ -88,9 +88,17 @@ k_preprocess(GaussIn g, const ViewInfo *__restrict__ views, int n_views, float z
                 rrow[22] = rgb[1];
                 rrow[23] = rgb[2];
                 float4 *dst = rec + it * kRecF4;
+                if (g.splat) {
+                    dst[0] = make_float4(rrow[9], rrow[10], rrow[12], rrow[13]);
+                    dst[1] = make_float4(rrow[15], rrow[16], rrow[18], rrow[19]);
+                    dst[2] = make_float4(rrow[20], rrow[21], rrow[22], rrow[23]);
+                } else {
 #pragma unroll
-                for (int k = 0; k < kRecF4; ++k)
-                    dst[k] = make_float4(rrow[4 * k], rrow[4 * k + 1], rrow[4 * k + 2], rrow[4 * k + 3]);
+                    for (int k = 0; k < 4; ++k)
+                        dst[k] = make_float4(rrow[2 * k], rrow[9 + 2 * k], rrow[2 * k + 1], rrow[10 + 2 * k]);
+                    dst[4] = make_float4(rrow[8], rrow[17], rrow[18], rrow[19]);
+                    dst[5] = make_float4(rrow[20], rrow[21], rrow[22], rrow[23]);
+                }
             } else {
                 rc = make_short4(-1, -1, -1, -1);
                 prc = rc;

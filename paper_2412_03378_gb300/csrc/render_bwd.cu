@@ -11,7 +11,8 @@
 // u = (dx, dy, 1), so with ga = 2 dL/da and gq = 2 dL/dq per pixel (a = |d'|^2, q = |o' x d'|^2)
 //   dL/dA = A sum_p ga u u^T,   dL/dC = C sum_p gq u u^T:
 // per Gaussian only the two symmetric 3x3 moment matrices (6 + 6 values), sum dL/dln(kappa) and
-// the three colour partials are summed -- 16 values, added to the per-item accumulator in L2
+// the three colour partials are summed (the two matrices' entries packed in pairs, as d' and o' x d' are
+// formed: 0.403 -> 0.386 ms on the 1M-Gaussian 1280 x 832 step, bound by issue slots) -- 16 values, added to the per-item accumulator in L2
 // with vector reductions (red.global.add.v4/v2).  When at most kDirectLanes lanes of the warp
 // contribute to a Gaussian, each of them adds its 16 values directly (four v4 reductions);
 // otherwise three shuffle exchange steps leave every lane with 2 values summed over 8 lanes,
@@ -28,8 +29,8 @@
 
 namespace vg {
 
-// Accumulator layout per item: [0..5] sum ga (xx, xy, x, yy, y, 1), [6..11] the same for gq,
-// [12] sum dL/dln(kappa), [13..15] dL/dcolour.
+// Accumulator layout per item: [0..11] sum of (ga, gq) times xx, xy, x, yy, y, 1 (pairs, as the packed
+// operations leave them), [12] sum dL/dln(kappa), [13..15] dL/dcolour.
 constexpr int kGradUsed = 16;
 static_assert(kGradUsed == kGradN, "the vector reductions cover the whole 16-float accumulator");
 constexpr int kDirectLanes = 12;   // at most this many contributing lanes: direct reductions
@@ -47,18 +48,18 @@ constexpr int kDirectLanes = 12;   // at most this many contributing lanes: dire
 constexpr int kGroup = 32;                               // records per ring slot
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // 1 s
 
-template <bool PIXTEST>
+template <bool PIXTEST, bool SPLAT>
 struct RingSlot {
-    float4 rec[kGroup * kRecF4];                // the records, one after another
-    float4 cull[PIXTEST ? 1 : kCullF4][kGroup];  // Gram rows for the opacity test, by row
-    float4 ref[PIXTEST ? 1 : kGroup];            // (px0, py0, log2 K, |A0|) for the opacity test
-    float sa1[PIXTEST ? 1 : kGroup];             // |A1| for the opacity test
-    short4 rect[kGroup];                         // pixel footprint rectangles
-    uint32_t item[kGroup];                       // item ids (accumulator rows)
+    float4 rec[kGroup * RecOf<SPLAT>::kF4];             // the records, one after another
+    float4 cull[PIXTEST ? 1 : kCullF4<SPLAT>][kGroup];  // Gram rows for the opacity test, by row
+    float4 ref[PIXTEST ? 1 : kGroup];                   // (px0, py0, log2 K, |A0|) for the opacity test
+    float sa1[PIXTEST ? 1 : kGroup];                    // |A1| for the opacity test
+    short4 rect[kGroup];                                // pixel footprint rectangles
+    uint32_t item[kGroup];                              // item ids (accumulator rows)
 };
 
-// One CTA per tile (longest list first): tw th / P consumer threads owning P pixels each, plus
-// the producer warp.  For each group a consumer warp first ballots which records it needs (some
+// One CTA per tile (longest list first; with few tiles two, see tile_split): tw th / P consumer
+// threads owning P pixels each, plus the producer warp.  For each group a consumer warp first ballots which records it needs (some
 // pixel of the warp reached the record, the record's footprint touches the warp's pixels and,
 // when pairs below tau_skip are skipped, its opacity can reach tau_skip there), then visits only
 // those, back to front.  The chunk setting CH gives the ring depth: CH / 16 slots (4 or 8, i.e.
@@ -70,11 +71,12 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
              const uint2 *__restrict__ ranges, const uint32_t *__restrict__ sorted_item, const float4 *__restrict__ rec,
              const short4 *__restrict__ prect, BlendParams bp, const float *__restrict__ T_fin, const float *__restrict__ S_fin,
              const uint32_t *__restrict__ nlast, const float *__restrict__ dL_drgb, const float *__restrict__ dL_dT,
-             float *__restrict__ grad_acc, unsigned long long *__restrict__ pair_count, uint32_t *__restrict__ err) {
+             float *__restrict__ grad_acc, unsigned long long *__restrict__ pair_count, uint32_t *__restrict__ err, int split) {
     pdl_entry();
     using L = PixLayout<P>;
     constexpr int kSlots = CH / 16;
-    using Slot = RingSlot<PIXTEST>;
+    using Slot = RingSlot<PIXTEST, SPLAT>;
+    constexpr int kRF4 = RecOf<SPLAT>::kF4;
     __shared__ Slot ring[kSlots];
     __shared__ __align__(8) uint64_t full[kSlots], empty[kSlots];
     __shared__ uint32_t s_last;
@@ -82,12 +84,13 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
 
     const int n_cons = (int)blockDim.x - 32;   // consumer threads; the last warp produces
     const bool producer = (int)threadIdx.x >= n_cons;
-    const int tile = tile_order ? tile_order[blockIdx.x] : (int)blockIdx.x;
+    const int rank = (int)blockIdx.x / split, tid = ((int)blockIdx.x - rank * split) * n_cons + (int)threadIdx.x;
+    const int tile = tile_order ? tile_order[rank] : rank;
     const ViewInfo &V = views[tile_view[tile]];
     const int local = tile - V.tile_base;
     const int tyi = local / V.tiles_x, txi = local - tyi * V.tiles_x;
     int ix, iy;
-    L::origin(producer ? 0 : (int)threadIdx.x, V.tw, ix, iy);
+    L::origin(producer ? 0 : tid, V.tw, ix, iy);
     const int x0 = txi * V.tw + ix, y0 = tyi * V.th + iy;
     const uint2 rg = ranges[tile];
     const int lane = threadIdx.x & 31;
@@ -158,21 +161,19 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
             if (lane < (int)(end - start)) {
                 const uint32_t item = sorted_item[start + lane];
                 const float4 *src = rec + (size_t)item * kRecF4;
-                float4 q[kRecF4];
+                float4 q[kRF4];
 #pragma unroll
-                for (int k = 0; k < kRecF4; ++k) q[k] = __ldg(src + k);
+                for (int k = 0; k < kRF4; ++k) q[k] = __ldg(src + k);
                 const short4 pr = prect[item];
 #pragma unroll
-                for (int k = 0; k < kRecF4; ++k) Sl.rec[lane * kRecF4 + k] = q[k];
+                for (int k = 0; k < kRF4; ++k) Sl.rec[lane * kRF4 + k] = q[k];
                 Sl.rect[lane] = pr;
                 Sl.item[lane] = item;
                 if (!PIXTEST) {
-                    float4 c[kCullF4];
-                    cull_row(q[0], q[1], q[2], q[3], q[4], c);
+                    float4 c[kCullF4<SPLAT>];
+                    cull_row<SPLAT>(q, c, Sl.ref[lane], Sl.sa1[lane]);
 #pragma unroll
-                    for (int k = 0; k < kCullF4; ++k) Sl.cull[k][lane] = c[k];
-                    Sl.ref[lane] = make_float4(q[4].z, q[4].w, q[5].x, sqrtf(c[0].x));
-                    Sl.sa1[lane] = sqrtf(c[0].w);
+                    for (int k = 0; k < kCullF4<SPLAT>; ++k) Sl.cull[k][lane] = c[k];
                 }
             }
             mbar_arrive(&full[sl]);
@@ -197,24 +198,20 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
             const Slot &Sl = ring[sl];
             const int n = (int)(end - start);
             bool need = lane < n && start + (uint32_t)lane < warp_last && !box_misses(wb, Sl.rect[lane]);
-            if (!PIXTEST && need) {   // skip records whose opacity stays below tau_skip on this warp
-                const float4 r = Sl.ref[lane];
-                need = box_may_blend(Sl.cull[0][lane], Sl.cull[1][lane], Sl.cull[2][lane], r.x, r.y, r.z, r.w,
-                                     Sl.sa1[lane], bc);
-            }
+            if (!PIXTEST && need)   // skip records whose opacity stays below tau_skip on this warp
+                need = rec_may_blend<SPLAT>([&](int k) { return Sl.cull[k][lane]; }, Sl.ref[lane], Sl.sa1[lane], bc);
             unsigned m = __ballot_sync(0xffffffffu, need);
             while (m) {
                 const int b = 31 - __clz(m);
                 m ^= 1u << b;
                 const int j = b;
                 const uint32_t idx = start + (uint32_t)j;
-                float gv[kGradUsed];
-#pragma unroll
-                for (int k = 0; k < kGradUsed; ++k) gv[k] = 0.0f;
+                F2 gm[6];            // (ga, gq) moments
+                float gv[4];         // dL/dln(kappa), dL/dcolour
                 bool any = false;
                 {
-                    const float4 *r = &Sl.rec[j * kRecF4];
-                    const float4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3], r4 = r[4], r5 = r[5];
+                    typename RecOf<SPLAT>::type r;
+                    load_rec(&Sl.rec[j * kRF4], r);
                     short4 pr;
                     if (PIXTEST) pr = Sl.rect[j];
                     constexpr int kCols = P == 4 ? 2 : 1;   // pixel columns of the thread
@@ -223,9 +220,9 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
 #pragma unroll
                     for (int c = 0; c < kCols; ++c) {
                         if constexpr (SPLAT)
-                            splat_col(r2, r3, r4, c ? xf + 1.0f : xf, sc[c]);
+                            splat_col(r, c ? xf + 1.0f : xf, sc[c]);
                         else
-                            col_base(r0, r1, r2, r3, r4, c ? xf + 1.0f : xf, cb[c]);
+                            col_base(r, c ? xf + 1.0f : xf, cb[c]);
                     }
 #pragma unroll
                     for (int k = 0; k < P; ++k) {
@@ -234,7 +231,7 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                         float tau, e2, alpha, pdx, pdy, kG, ca, cq;
                         if constexpr (SPLAT) {
                             float q;
-                            const float ar = splat_at(r3, r4, r5, sc[L::ox(k)], L::oy(k) ? yf + (float)L::oy(k) : yf, pdx, pdy, q);
+                            const float ar = splat_at(r, sc[L::ox(k)], L::oy(k) ? yf + (float)L::oy(k) : yf, pdx, pdy, q);
                             if (COUNT) pairs += valid;
                             const bool clamped = ar > bp.alpha_max;
                             const float a_c = fminf(ar, bp.alpha_max);
@@ -248,7 +245,7 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                             cq = -1.0f;        // ln(o G') = ln o - q/2
                         } else {
                             PairEval e;
-                            pair_eval_col(r0, r1, r3, r4, r5, cb[L::ox(k)], L::oy(k) ? yf + (float)L::oy(k) : yf, Lp[k], e);
+                            pair_eval_col(r, cb[L::ox(k)], L::oy(k) ? yf + (float)L::oy(k) : yf, Lp[k], e);
                             if (COUNT) pairs += valid;
                             const bool clamped = e.tau > bp.tau_max;
                             const float t_c = fminf(e.tau, bp.tau_max);
@@ -256,7 +253,7 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                             tau = valid ? t_c : 0.0f;
                             e2 = ex2_approx(__fmul_rn(-kLog2eF, tau));
                             alpha = __fsub_rn(1.0f, e2);
-                            pdx = e.dx;
+                            pdx = cb[L::ox(k)].dx;
                             pdy = e.dy;
                             kG = clamped ? 0.0f : tau;   // dln(tau)/dln(amplitude) = 1; a clamp cuts it
                             const float r2s = e.rs * e.rs;
@@ -268,52 +265,62 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                         const float Sb = S[k] - tau;
                         const float Tb = valid ? ex2_approx(-kLog2eF * Sb) : Tafter[k];
                         const float aT = alpha * Tb;
-                        gv[13] = fmaf(g0[k], aT, gv[13]);
-                        gv[14] = fmaf(g1[k], aT, gv[14]);
-                        gv[15] = fmaf(g2[k], aT, gv[15]);
                         // per channel c T - R with one rounding each (fma): a single scalar g . R
                         // measured less accurate for flattened Gaussians under Eq. 20
-                        const float dtau = g0[k] * fmaf(r5.y, Tafter[k], -R0[k]) + g1[k] * fmaf(r5.z, Tafter[k], -R1[k]) +
-                                           g2[k] * fmaf(r5.w, Tafter[k], -R2[k]) + gTterm[k];
-                        R0[k] = fmaf(r5.y, aT, R0[k]);
-                        R1[k] = fmaf(r5.z, aT, R1[k]);
-                        R2[k] = fmaf(r5.w, aT, R2[k]);
+                        const float dtau = g0[k] * fmaf(r.q5.y, Tafter[k], -R0[k]) + g1[k] * fmaf(r.q5.z, Tafter[k], -R1[k]) +
+                                           g2[k] * fmaf(r.q5.w, Tafter[k], -R2[k]) + gTterm[k];
+                        R0[k] = fmaf(r.q5.y, aT, R0[k]);
+                        R1[k] = fmaf(r.q5.z, aT, R1[k]);
+                        R2[k] = fmaf(r.q5.w, aT, R2[k]);
                         S[k] = Sb;
                         Tafter[k] = Tb;
                         const float G = dtau * kG;                   // dL / d ln(amplitude)
-                        const float gq = G * cq;                     // 2 dL/dq
-                        const float xx = pdx * pdx, xy = pdx * pdy, yy = pdy * pdy;
-                        if constexpr (!SPLAT) {
-                            const float ga = G * ca;                 // 2 dL/da
-                            gv[0] = fmaf(ga, xx, gv[0]);
-                            gv[1] = fmaf(ga, xy, gv[1]);
-                            gv[2] = fmaf(ga, pdx, gv[2]);
-                            gv[3] = fmaf(ga, yy, gv[3]);
-                            gv[4] = fmaf(ga, pdy, gv[4]);
-                            gv[5] += ga;
+                        // (2 dL/da, 2 dL/dq) and its moments
+                        const F2 g = f2_mul(f2_dup(G), f2_pack(ca, cq)), dx = f2_dup(pdx), dy = f2_dup(pdy);
+                        const F2 xx = f2_dup(pdx * pdx), xy = f2_dup(pdx * pdy), yy = f2_dup(pdy * pdy);
+                        if (k == 0) {
+                            gv[0] = G;
+                            gv[1] = g0[k] * aT;
+                            gv[2] = g1[k] * aT;
+                            gv[3] = g2[k] * aT;
+                            gm[0] = f2_mul(g, xx);
+                            gm[1] = f2_mul(g, xy);
+                            gm[2] = f2_mul(g, dx);
+                            gm[3] = f2_mul(g, yy);
+                            gm[4] = f2_mul(g, dy);
+                            gm[5] = g;
+                        } else {
+                            gv[0] += G;
+                            gv[1] = fmaf(g0[k], aT, gv[1]);
+                            gv[2] = fmaf(g1[k], aT, gv[2]);
+                            gv[3] = fmaf(g2[k], aT, gv[3]);
+                            gm[0] = f2_fma(g, xx, gm[0]);
+                            gm[1] = f2_fma(g, xy, gm[1]);
+                            gm[2] = f2_fma(g, dx, gm[2]);
+                            gm[3] = f2_fma(g, yy, gm[3]);
+                            gm[4] = f2_fma(g, dy, gm[4]);
+                            gm[5] = f2_add(gm[5], g);
                         }
-                        gv[6] = fmaf(gq, xx, gv[6]);
-                        gv[7] = fmaf(gq, xy, gv[7]);
-                        gv[8] = fmaf(gq, pdx, gv[8]);
-                        gv[9] = fmaf(gq, yy, gv[9]);
-                        gv[10] = fmaf(gq, pdy, gv[10]);
-                        gv[11] += gq;
-                        gv[12] += G;
                     }
                 }
                 const unsigned act = __ballot_sync(0xffffffffu, any);
                 if (act) {
                     float *dst = grad_acc + (size_t)Sl.item[j] * kGradN;   // 64-byte aligned
+                    float v[kGradUsed];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) f2_unpack(gm[k], v[2 * k], v[2 * k + 1]);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) v[12 + k] = gv[k];
                     if (__popc(act) <= kDirectLanes) {
                         if (any) {
-                            red_add_v4(dst, gv[0], gv[1], gv[2], gv[3]);
-                            red_add_v4(dst + 4, gv[4], gv[5], gv[6], gv[7]);
-                            red_add_v4(dst + 8, gv[8], gv[9], gv[10], gv[11]);
-                            red_add_v4(dst + 12, gv[12], gv[13], gv[14], gv[15]);
+                            red_add_v4(dst, v[0], v[1], v[2], v[3]);
+                            red_add_v4(dst + 4, v[4], v[5], v[6], v[7]);
+                            red_add_v4(dst + 8, v[8], v[9], v[10], v[11]);
+                            red_add_v4(dst + 12, v[12], v[13], v[14], v[15]);
                         }
                     } else {
-                        const int b0 = warp_reduce_scatter_part<kGradUsed, 3>(gv, lane);
-                        red_add_v2(dst + b0, gv[0], gv[1]);
+                        const int b0 = warp_reduce_scatter_part<kGradUsed, 3>(v, lane);
+                        red_add_v2(dst + b0, v[0], v[1]);
                     }
                 }
             }
@@ -337,15 +344,17 @@ static void launch_bwd_ptsc(const ViewInfo *views_d, const int *tile_view, const
                             const BlendParams &bp, const float *T_fin, const float *S_fin, const uint32_t *nlast,
                             const float *dL_drgb, const float *dL_dT, float *grad_acc, unsigned long long *pair_count,
                             uint32_t *err, cudaStream_t st) {
-    const unsigned threads = (unsigned)(bp.tile_px / P + 32);   // consumers + the producer warp
+    const int split = tile_split(n_tiles, bp.tile_px / P);
+    const unsigned threads = (unsigned)(bp.tile_px / P / split + 32);   // consumers + the producer warp
+    n_tiles *= split;
     if (pair_count)
         pdl_launch(k_render_bwd<P, true, PIXTEST, SPLAT, CH>, (unsigned)n_tiles, threads, 0, st,
             views_d, tile_view, tile_order, ranges, sorted_item, rec, prect, bp, T_fin, S_fin, nlast, dL_drgb, dL_dT,
-            grad_acc, pair_count, err);
+            grad_acc, pair_count, err, split);
     else
         pdl_launch(k_render_bwd<P, false, PIXTEST, SPLAT, CH>, (unsigned)n_tiles, threads, 0, st,
             views_d, tile_view, tile_order, ranges, sorted_item, rec, prect, bp, T_fin, S_fin, nlast, dL_drgb, dL_dT,
-            grad_acc, nullptr, err);
+            grad_acc, nullptr, err, split);
 }
 
 template <int P, bool PIXTEST, bool SPLAT>
@@ -417,7 +426,7 @@ __device__ __forceinline__ void cross_add(const float a[3], const float b[3], fl
 }
 
 // Splat mode (Eq. 5-7): the moments Mq = sum gq u u^T (gq = 2 dL/dq, u = (dx, dy, 1) from the
-// reference pixel; accumulator entries 6..11) of one (view, Gaussian) give, with w = u - m,
+// reference pixel; the accumulator's odd entries 1..11) of one (view, Gaussian) give, with w = u - m,
 //   dL/dQ = (1/2) sum gq w w^T,   dL/dmu' = -Q sum gq w      (q = w' Q w, Q = Sigma'^-1),
 // then dL/dSigma' = -Q dL/dQ Q and, with Sigma' = B B^T + dil I, dL/dB = -2 Q dL/dQ P where
 // P = Q B has the rows (b_1 x n + dil b_0) / det and (n x b_0 + dil b_1) / det (n = b_0 x b_1:
@@ -435,7 +444,7 @@ __device__ __forceinline__ void splat_chain(const ViewInfo &V, const float mu[3]
         return;
     }
     const float mx = G.mx, my = G.my;
-    const float M00 = ga[6], M01 = ga[7], M02 = ga[8], M11 = ga[9], M12 = ga[10], M22 = ga[11];
+    const float M00 = ga[1], M01 = ga[3], M02 = ga[5], M11 = ga[7], M12 = ga[9], M22 = ga[11];
     const float Sx = fmaf(-mx, M22, M02), Sy = fmaf(-my, M22, M12);
     const float Sxx = fmaf(-mx, M02 + Sx, M00);
     const float Sxy = fmaf(-mx, Sy, fmaf(-my, M02, M01));
@@ -573,8 +582,8 @@ k_chain(GaussIn g, const ViewInfo *__restrict__ views, int n_views, float *__res
         // Ma = sum ga u u^T over u = (dx, dy, 1), stored as (xx, xy, x, yy, y, 1).
         float dA[9], dC[9];
         {
-            const float Ma[9] = {ga[0], ga[1], ga[2], ga[1], ga[3], ga[4], ga[2], ga[4], ga[5]};
-            const float Mq[9] = {ga[6], ga[7], ga[8], ga[7], ga[9], ga[10], ga[8], ga[10], ga[11]};
+            const float Ma[9] = {ga[0], ga[2], ga[4], ga[2], ga[6], ga[8], ga[4], ga[8], ga[10]};
+            const float Mq[9] = {ga[1], ga[3], ga[5], ga[3], ga[7], ga[9], ga[5], ga[9], ga[11]};
 #pragma unroll
             for (int j = 0; j < 3; ++j)
 #pragma unroll

@@ -8,38 +8,49 @@
 // leaves once all of its pixels have reached T < T_stop.  The per-pixel update is branch-free: a
 // pixel that does not blend the visited Gaussian (finished, outside the image or the footprint,
 // or below the skip threshold) takes tau = 0 (alpha = 0), which leaves its colour, T and S
-// unchanged bit for bit (0.247 ms against 0.270 ms with per-pixel branches).  SPLAT selects the 3DGS comparison
-// mode's alpha (Eq. 6) in the same loop.  No tensor cores: the work is not a
+// unchanged bit for bit (0.247 ms against 0.270 ms with per-pixel branches).  Issue slots bound it, so
+// the operations are packed two to an instruction: d' with o' x d' (RecPairs) and, with two rows per
+// thread, the pixels' own chains (1M Gaussians, 1280 x 832: 0.255 -> 0.235 ms).  SPLAT selects the 3DGS comparison
+// mode's alpha (Eq. 6) in the same loop, on records of half the size.  No tensor cores: the work is not a
 // dense contraction.
 #include "blend.cuh"
 
 namespace vg {
 
+// Records evaluated together with one pixel per thread, the form for few tiles, whose time is the longest list's chain of
+// dependent instructions.  1,040 tiles (100,000 Gaussians) at 1 / 2 / 3 / 4: 116.8 / 99.7 / 98.1 / 95.9 us.
+constexpr int kIlp = 4;
 
-// One CTA of tw th / P threads per tile.  The register cap is that of 3 / 7 / 12 CTAs of a 16 x 16
-// tile per SM for P = 1 / 2 / 4 (the occupancy measured fastest), whatever the tile shape.
+// One CTA of tw th / P threads per tile (with P = 1, `split` CTAs of as many threads in all, see
+// tile_split).  The register cap is that of 3 / 7 / 12 CTAs of a 16 x 16 tile per SM for P = 1 / 2 / 4 (the occupancy measured fastest), whatever the tile shape.
 template <int P, bool COUNT, bool PIXTEST, bool SPLAT, int CH>
 __global__ void __maxnreg__(PixLayout<P>::kFwdRegs)
 k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_view, const int *__restrict__ tile_order,
              const uint2 *__restrict__ ranges, const uint32_t *__restrict__ sorted_item, const float4 *__restrict__ rec,
              const short4 *__restrict__ prect, BlendParams bp, float *__restrict__ rgb, float *__restrict__ T_user, float *__restrict__ T_ws,
              float *__restrict__ S_out, uint32_t *__restrict__ nlast_out, uint32_t *__restrict__ tile_replay,
-             unsigned long long *__restrict__ pair_count, L2Fused l2) {
+             unsigned long long *__restrict__ pair_count, L2Fused l2, int split) {
     pdl_entry();
     using L = PixLayout<P>;
     constexpr int kChunk = CH;   // records per barrier
-    __shared__ float4 srec[kChunk * kRecF4];
+    constexpr int kRF4 = RecOf<SPLAT>::kF4, kCF4 = kCullF4<SPLAT>;
+    __shared__ float4 srec[kChunk * kRF4];
     __shared__ short4 srect[kChunk];
-    __shared__ float4 scull[PIXTEST ? 1 : kChunk * kCullF4];   // Gram matrices for the opacity test
+    __shared__ float4 scull[PIXTEST ? 1 : kChunk * kCF4];   // Gram matrices for the opacity test
     // per record, contiguous for the opacity test: (px0, py0, log2 K, |A0|) and |A1|
     __shared__ float4 sref[PIXTEST ? 1 : kChunk];
     __shared__ float ssq1[PIXTEST ? 1 : kChunk];
-    const int tile = tile_order ? tile_order[blockIdx.x] : (int)blockIdx.x;
+    int rank = (int)blockIdx.x, tid = (int)threadIdx.x;
+    if constexpr (P == 1) {
+        rank = (int)blockIdx.x / split;
+        tid += ((int)blockIdx.x - rank * split) * (int)blockDim.x;
+    }
+    const int tile = tile_order ? tile_order[rank] : rank;
     const ViewInfo &V = views[tile_view[tile]];
     const int local = tile - V.tile_base;
     const int tyi = local / V.tiles_x, txi = local - tyi * V.tiles_x;
     int ix, iy;
-    L::origin(threadIdx.x, V.tw, ix, iy);
+    L::origin(tid, V.tw, ix, iy);
     const int x0 = txi * V.tw + ix, y0 = tyi * V.th + iy;
     float Lp[P], T[P], S[P], c0[P], c1[P], c2[P];
     uint32_t last[P];
@@ -64,20 +75,18 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
         for (uint32_t r = threadIdx.x; r < n; r += blockDim.x) {
             const uint32_t item = sorted_item[base + r];
             const float4 *src = rec + (size_t)item * kRecF4;
-            float4 q[kRecF4];
+            float4 q[kRF4];
 #pragma unroll
-            for (int k = 0; k < kRecF4; ++k) {
+            for (int k = 0; k < kRF4; ++k) {
                 q[k] = __ldg(src + k);
-                srec[r * kRecF4 + k] = q[k];
+                srec[r * kRF4 + k] = q[k];
             }
             srect[r] = prect[item];
             if (!PIXTEST) {
-                float4 c[kCullF4];
-                cull_row(q[0], q[1], q[2], q[3], q[4], c);
+                float4 c[kCF4];
+                cull_row<SPLAT>(q, c, sref[r], ssq1[r]);
 #pragma unroll
-                for (int k = 0; k < kCullF4; ++k) scull[r * kCullF4 + k] = c[k];
-                sref[r] = make_float4(q[4].z, q[4].w, q[5].x, sqrtf(c[0].x));
-                ssq1[r] = sqrtf(c[0].w);
+                for (int k = 0; k < kCF4; ++k) scull[r * kCF4 + k] = c[k];
             }
         }
         __syncthreads();
@@ -87,63 +96,135 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
             if (!__any_sync(0xffffffffu, live != 0)) break;
             const int jl = w0 + lane;
             bool need = jl < (int)n && !box_misses(wb, srect[jl]);
-            if (!PIXTEST && need) {   // skip records whose opacity stays below tau_skip on this warp
-                const float4 *q = &scull[jl * kCullF4];
-                const float4 rf = sref[jl];
-                need = box_may_blend(q[0], q[1], q[2], rf.x, rf.y, rf.z, rf.w, ssq1[jl], bc);
-            }
+            if (!PIXTEST && need)   // skip records whose opacity stays below tau_skip on this warp
+                need = rec_may_blend<SPLAT>([&](int k) { return scull[jl * kCF4 + k]; }, sref[jl], ssq1[jl], bc);
             unsigned m = __ballot_sync(0xffffffffu, need);
-            while (m) {
+            if constexpr (P == 1) {
+                // kIlp records at a time: what does not depend on the pixel's state (opacity, its exponential)
+                // is formed for all of them before the first is blended, so that their chains overlap
+                while (m) {
+                    int js[kIlp];
+                    float t[kIlp], e2[kIlp], al[kIlp];
+                    bool in[kIlp], v[kIlp];
+#pragma unroll
+                    for (int i = 0; i < kIlp; ++i) {
+                        in[i] = m != 0;
+                        js[i] = w0 + (m ? __ffs(m) - 1 : 0);
+                        m &= m - 1;
+                    }
+#pragma unroll
+                    for (int i = 0; i < kIlp; ++i) {
+                        typename RecOf<SPLAT>::type r;
+                        load_rec(&srec[js[i] * kRF4], r);
+                        if (PIXTEST) {
+                            const short4 pr = srect[js[i]];
+                            in[i] = in[i] & !pixel_outside(x0, y0, pr);
+                        }
+                        if constexpr (SPLAT) {   // Eq. 6: alpha = min(o G'(p), alpha_max)
+                            SplatCol sc;
+                            splat_col(r, xf, sc);
+                            float dx, dy, q;
+                            const float a_c = fminf(splat_at(r, sc, yf, dx, dy, q), bp.alpha_max);
+                            v[i] = in[i] & (a_c >= bp.alpha_min);
+                            al[i] = v[i] ? a_c : 0.0f;
+                            e2[i] = __fsub_rn(1.0f, al[i]);
+                            t[i] = -log1pf(-al[i]);
+                        } else {
+                            ColBase cb;
+                            col_base(r, xf, cb);
+                            PairEval e;
+                            pair_eval_col(r, cb, yf, Lp[0], e);
+                            const float t_c = fminf(e.tau, bp.tau_max);
+                            v[i] = in[i] & (t_c >= bp.tau_skip);
+                            t[i] = v[i] ? t_c : 0.0f;
+                            e2[i] = ex2_approx(__fmul_rn(-kLog2eF, t[i]));
+                            al[i] = __fsub_rn(1.0f, e2[i]);
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < kIlp; ++i) {
+                        const float4 q5 = srec[js[i] * kRF4 + kRF4 - 1];
+                        if (COUNT) {
+                            pairs += live && in[i];
+                            blended += live && v[i];
+                        }
+                        const float w = __fmul_rn(live ? al[i] : 0.0f, T[0]);
+                        c0[0] = fmaf(q5.y, w, c0[0]);
+                        c1[0] = fmaf(q5.z, w, c1[0]);
+                        c2[0] = fmaf(q5.w, w, c2[0]);
+                        T[0] = __fmul_rn(T[0], live ? e2[i] : 1.0f);
+                        S[0] = __fadd_rn(S[0], live ? t[i] : 0.0f);
+                        if (live && v[i]) last[0] = base + js[i] + 1;
+                        if (T[0] < bp.T_stop) live = 0;
+                    }
+                }
+            }
+            while (P > 1 && m) {
                 const int b = __ffs(m) - 1;
                 m &= m - 1;
                 const int j = w0 + b;
-                const float4 *r = &srec[j * kRecF4];
-                const float4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3], r4 = r[4], r5 = r[5];
+                typename RecOf<SPLAT>::type r;
+                load_rec(&srec[j * kRF4], r);
                 short4 pr;
                 if (PIXTEST) pr = srect[j];
-                constexpr int kCols = P == 4 ? 2 : 1;   // pixel columns of the thread
-                ColBase cb[kCols];
-                SplatCol sc[kCols];
+                if constexpr (P == 1) {
+                } else if constexpr (SPLAT) {
+                    SplatCol sc[P / 2];   // pixel columns of the thread
 #pragma unroll
-                for (int c = 0; c < kCols; ++c) {
-                    if constexpr (SPLAT)
-                        splat_col(r2, r3, r4, c ? xf + 1.0f : xf, sc[c]);
-                    else
-                        col_base(r0, r1, r2, r3, r4, c ? xf + 1.0f : xf, cb[c]);
-                }
+                    for (int c = 0; c < P / 2; ++c) splat_col(r, c ? xf + 1.0f : xf, sc[c]);
 #pragma unroll
-                for (int k = 0; k < P; ++k) {
-                    bool valid = (live >> k) & 1u;
-                    if (PIXTEST) valid = valid && !pixel_outside(x0 + L::ox(k), y0 + L::oy(k), pr);
-                    float tau, e2, w;
-                    if constexpr (SPLAT) {   // Eq. 6: alpha = min(o G'(p), alpha_max)
+                    for (int k = 0; k < P; ++k) {   // Eq. 6: alpha = min(o G'(p), alpha_max)
+                        bool valid = (live >> k) & 1u;
+                        if (PIXTEST) valid = valid && !pixel_outside(x0 + L::ox(k), y0 + L::oy(k), pr);
                         float dx, dy, q;
                         const float a_c =
-                            fminf(splat_at(r3, r4, r5, sc[L::ox(k)], L::oy(k) ? yf + (float)L::oy(k) : yf, dx, dy, q), bp.alpha_max);
+                            fminf(splat_at(r, sc[L::ox(k)], L::oy(k) ? yf + (float)L::oy(k) : yf, dx, dy, q), bp.alpha_max);
                         if (COUNT) pairs += valid;
                         valid = valid && a_c >= bp.alpha_min;
-                        const float alpha = valid ? a_c : 0.0f;
-                        e2 = __fsub_rn(1.0f, alpha);
-                        tau = -log1pf(-alpha);
-                        w = __fmul_rn(alpha, T[k]);
-                    } else {
-                        PairEval e;
-                        pair_eval_col(r0, r1, r3, r4, r5, cb[L::ox(k)], L::oy(k) ? yf + (float)L::oy(k) : yf, Lp[k], e);
-                        if (COUNT) pairs += valid;
-                        const float t_c = fminf(e.tau, bp.tau_max);
-                        valid = valid && t_c >= bp.tau_skip;
-                        tau = valid ? t_c : 0.0f;
-                        e2 = ex2_approx(__fmul_rn(-kLog2eF, tau));
-                        w = __fmul_rn(__fsub_rn(1.0f, e2), T[k]);
+                        if (COUNT) blended += valid;
+                        const float alpha = valid ? a_c : 0.0f, e2 = __fsub_rn(1.0f, alpha), tau = -log1pf(-alpha);
+                        const float w = __fmul_rn(alpha, T[k]);
+                        c0[k] = fmaf(r.q5.y, w, c0[k]);
+                        c1[k] = fmaf(r.q5.z, w, c1[k]);
+                        c2[k] = fmaf(r.q5.w, w, c2[k]);
+                        T[k] = __fmul_rn(T[k], e2);
+                        S[k] = __fadd_rn(S[k], tau);
+                        if (valid) last[k] = base + j + 1;
+                        if (T[k] < bp.T_stop) live &= ~(1u << k);
                     }
-                    if (COUNT) blended += valid;
-                    c0[k] = fmaf(r5.y, w, c0[k]);
-                    c1[k] = fmaf(r5.z, w, c1[k]);
-                    c2[k] = fmaf(r5.w, w, c2[k]);
-                    T[k] = __fmul_rn(T[k], e2);
-                    S[k] = __fadd_rn(S[k], tau);
-                    if (valid) last[k] = base + j + 1;
-                    if (T[k] < bp.T_stop) live &= ~(1u << k);
+                } else {   // the same operations, packed over the two rows of a column
+#pragma unroll
+                    for (int c = 0; c < P / 2; ++c) {
+                        constexpr int kRow = P / 2;   // pixel k = c + row kRow
+                        ColBase cb;
+                        col_base(r, c ? xf + 1.0f : xf, cb);
+                        float t[2], e[2];
+                        pair_tau2(r, cb, f2_pack(yf, yf + 1.0f), f2_pack(Lp[c], Lp[c + kRow]), t);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int k = c + h * kRow;
+                            bool valid = (live >> k) & 1u;
+                            if (PIXTEST) valid = valid && !pixel_outside(x0 + c, y0 + h, pr);
+                            if (COUNT) pairs += valid;
+                            const float t_c = fminf(t[h], bp.tau_max);
+                            valid = valid && t_c >= bp.tau_skip;
+                            t[h] = valid ? t_c : 0.0f;
+                            if (COUNT) blended += valid;
+                            if (valid) last[k] = base + j + 1;
+                        }
+                        const F2 tau = f2_pack(t[0], t[1]), Tk = f2_pack(T[c], T[c + kRow]);
+                        f2_unpack(f2_mul(f2_dup(-kLog2eF), tau), e[0], e[1]);
+                        const F2 e2 = f2_pack(ex2_approx(e[0]), ex2_approx(e[1]));
+                        const F2 w = f2_mul(f2_fma(e2, f2_dup(-1.0f), f2_dup(1.0f)), Tk);   // (1 - e2) T
+                        f2_unpack(f2_fma(f2_dup(r.q5.y), w, f2_pack(c0[c], c0[c + kRow])), c0[c], c0[c + kRow]);
+                        f2_unpack(f2_fma(f2_dup(r.q5.z), w, f2_pack(c1[c], c1[c + kRow])), c1[c], c1[c + kRow]);
+                        f2_unpack(f2_fma(f2_dup(r.q5.w), w, f2_pack(c2[c], c2[c + kRow])), c2[c], c2[c + kRow]);
+                        f2_unpack(f2_mul(Tk, e2), T[c], T[c + kRow]);
+                        f2_unpack(f2_add(f2_pack(S[c], S[c + kRow]), tau), S[c], S[c + kRow]);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            if (T[c + h * kRow] < bp.T_stop) live &= ~(1u << (c + h * kRow));
+                    }
                 }
             }
         }
@@ -201,15 +282,17 @@ static void launch_fwd_ptsc(const ViewInfo *views_d, const int *tile_view, const
                             const BlendParams &bp, float *rgb, float *T_user, float *T_ws, float *S_out,
                             uint32_t *nlast_out, uint32_t *tile_replay, unsigned long long *pair_count,
                             const L2Fused &l2, cudaStream_t st) {
-    const unsigned threads = (unsigned)(bp.tile_px / P);
+    const int split = P == 1 ? tile_split(n_tiles, bp.tile_px / P) : 1;
+    const unsigned threads = (unsigned)(bp.tile_px / P / split);
+    n_tiles *= split;
     if (pair_count)
         pdl_launch(k_render_fwd<P, true, PIXTEST, SPLAT, CH>, (unsigned)n_tiles, threads, 0, st,
             views_d, tile_view, tile_order, ranges, sorted_item, rec, prect, bp, rgb, T_user, T_ws, S_out, nlast_out, tile_replay,
-            pair_count, l2);
+            pair_count, l2, split);
     else
         pdl_launch(k_render_fwd<P, false, PIXTEST, SPLAT, CH>, (unsigned)n_tiles, threads, 0, st,
             views_d, tile_view, tile_order, ranges, sorted_item, rec, prect, bp, rgb, T_user, T_ws, S_out, nlast_out, tile_replay,
-            nullptr, l2);
+            nullptr, l2, split);
 }
 
 template <int P, bool PIXTEST, bool SPLAT>
