@@ -64,6 +64,7 @@ struct vg_workspace {
     DBuf<short4> vbox;                    // voxel query: truncation boxes (2 per Gaussian)
     DBuf<float4> march_E;                 // ray march: o'.A_k per item
     DBuf<float4> march_part;              // ray march: colour and transmittance per (group of passes, pixel)
+    DBuf<float> cone_w;                   // cone-beam backward: pixel weights
     DBuf<float> tomo_dl;                  // tomography backward: dL/dtau of one angle batch's pixels, padded rows
     uint32_t *tile_order = nullptr;       // longest-first tile order of the last bin_sort
     uint32_t *tile_order_bwd = nullptr;   // longest replay first, from the last forward (NULL: none)
@@ -292,6 +293,7 @@ vg_status vg_workspace_destroy(vg_workspace *ws) {
     release(ws->vbox);
     release(ws->march_E);
     release(ws->march_part);
+    release(ws->cone_w);
     release(ws->tomo_dl);
     if (ws->h_total) cudaFreeHost(ws->h_total);
     for (auto &r : ws->prof) {
@@ -690,11 +692,12 @@ vg_status vg_render_fwd_l2(vg_workspace *ws, float *rgb, float *T_final, const f
         VG_CUDA(ws, cudaMemsetAsync(loss, 0, sizeof(float), (cudaStream_t)stream));
         return render_fwd_impl(ws, rgb, T_final, stream, false);
     }
-    return render_fwd_impl(ws, rgb, T_final, stream, false, L2Fused{target, dL_drgb, loss, scale});
+    return render_fwd_impl(ws, rgb, T_final, stream, false, L2Fused{target, dL_drgb, loss, scale, nullptr, nullptr});
 }
 
 static vg_status render_bwd_impl(vg_workspace *ws, const float *dL_drgb, const float *dL_dT, float *dmu, float *dscale,
-                                 float *dquat, float *dkappa, float *dsh, void *stream, bool drgb_optional) {
+                                 float *dquat, float *dkappa, float *dsh, void *stream, bool drgb_optional,
+                                 const float *cone_weights = nullptr) {
     if (!ws) return VG_ERR_INVALID_ARG;
     if (ws->stage < 3) return fail(ws, VG_ERR_STATE, "vg_render_bwd before vg_render_fwd");
     if ((!dL_drgb && ws->n_pixels > 0 && !drgb_optional) || (ws->g.n > 0 && (!dmu || !dscale || !dquat || !dkappa)))
@@ -712,7 +715,11 @@ static vg_status render_bwd_impl(vg_workspace *ws, const float *dL_drgb, const f
     }
     {
         ProfScope ps(ws, ST_BWD, st);
-        VG_CUDA(ws, launch_render_bwd(ws->views.p, ws->tile_view.p, (const int *)bwd_order(ws), ws->n_tiles,
+        if (cone_weights)
+            VG_CUDA(ws, launch_cone_bwd(ws->views.p, ws->n_items, ws->g.n, ws->rec.p, ws->prect.p, cone_weights, ws->grad.p,
+                                        st, &ws->launches));
+        else
+            VG_CUDA(ws, launch_render_bwd(ws->views.p, ws->tile_view.p, (const int *)bwd_order(ws), ws->n_tiles,
                                       ws->ranges.p, ws->inst_item, ws->rec.p, ws->prect.p, ws->bp, ws->ppt_bwd,
                                       ws->T_fin.p,
                                       ws->S_fin.p, ws->nlast.p, dL_drgb, dL_dT, ws->grad.p, pc, lookback_err_ptr(ws),
@@ -754,8 +761,23 @@ vg_status vg_project_cone(vg_workspace *ws, const vg_gaussians *g, const vg_came
     VG_TRY(preprocess_impl(ws, g ? &gd : nullptr, cams, n_views, &o, stream, false));
     VG_TRY(vg_bin_sort(ws, stream));
     if (!proj && ws->n_pixels > 0) return fail(ws, VG_ERR_INVALID_ARG, "proj is NULL");
-    VG_TRY(render_fwd_impl(ws, nullptr, proj, stream, true));
-    if (dL_dproj) VG_TRY(render_bwd_impl(ws, nullptr, dL_dproj, dmu, dscale, dquat, dkappa, nullptr, stream, true));
+    // The gradient item by item from pixel weights that the forward writes.  Where their buffer is missing and may
+    // not be allocated (fixed capacity, a capturing stream), and when pairs are counted, the blend's backward runs.
+    bool by_item = dL_dproj && !(opts->flags & VG_FLAG_COUNT_PAIRS);
+    if (by_item && (!ws->cone_w.p || ws->cone_w.n < (size_t)ws->n_pixels)) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        VG_CUDA(ws, cudaStreamIsCapturing((cudaStream_t)stream, &cap));
+        if (cap != cudaStreamCaptureStatusNone || (ws->cone_w.p && (opts->flags & VG_FLAG_FIXED_CAPACITY)))
+            by_item = false;
+        else
+            VG_TRY(ensure(ws, ws->cone_w, (size_t)ws->n_pixels, "pixel weights"));
+    }
+    L2Fused ep{};
+    if (by_item) ep.dproj = dL_dproj, ep.weights = ws->cone_w.p;
+    VG_TRY(render_fwd_impl(ws, nullptr, proj, stream, true, ep));
+    if (dL_dproj)
+        VG_TRY(render_bwd_impl(ws, nullptr, dL_dproj, dmu, dscale, dquat, dkappa, nullptr, stream, true,
+                               by_item ? ws->cone_w.p : nullptr));
     return VG_OK;
 }
 

@@ -18,12 +18,16 @@
 namespace vg {
 
 // Records evaluated together with one pixel per thread, the form for few tiles, whose time is the longest list's chain of
-// dependent instructions.  1,040 tiles (100,000 Gaussians) at 1 / 2 / 3 / 4: 116.8 / 99.7 / 98.1 / 95.9 us.
+// dependent instructions.  1,040 tiles (100,000 Gaussians) at 1 / 2 / 3 / 4: 116.8 / 99.7 / 98.1 / 95.9 us.  With two
+// pixels per thread one record at a time, and two where every footprint pixel counts (3,584 tiles, no skip: 926 / 812 us;
+// with the skip's shorter visits 229 / 235 us on the 1M-Gaussian 1280 x 832 workload).
 constexpr int kIlp = 4;
+// volumetric blend, the 3DGS comparison mode, cone-beam projection (rgb NULL, nothing skipped, clamped or stopped)
+constexpr int kModeBlend = 0, kModeSplat = 1, kModeCone = 2;
 
 // One CTA of tw th / P threads per tile (with P = 1, `split` CTAs of as many threads in all, see
 // tile_split).  The register cap is that of 3 / 7 / 12 CTAs of a 16 x 16 tile per SM for P = 1 / 2 / 4 (the occupancy measured fastest), whatever the tile shape.
-template <int P, bool COUNT, bool PIXTEST, bool SPLAT, int CH>
+template <int P, bool COUNT, bool PIXTEST, int MODE, int CH>
 __global__ void __maxnreg__(PixLayout<P>::kFwdRegs)
 k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_view, const int *__restrict__ tile_order,
              const uint2 *__restrict__ ranges, const uint32_t *__restrict__ sorted_item, const float4 *__restrict__ rec,
@@ -32,6 +36,7 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
              unsigned long long *__restrict__ pair_count, L2Fused l2, int split) {
     pdl_entry();
     using L = PixLayout<P>;
+    constexpr bool SPLAT = MODE == kModeSplat, CONE = MODE == kModeCone;
     constexpr int kChunk = CH;   // records per barrier
     constexpr int kRF4 = RecOf<SPLAT>::kF4, kCF4 = kCullF4<SPLAT>;
     __shared__ float4 srec[kChunk * kRF4];
@@ -148,6 +153,11 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                             pairs += live && in[i];
                             blended += live && v[i];
                         }
+                        if constexpr (CONE) {   // the sum of tau is all the projection needs
+                            S[0] = __fadd_rn(S[0], live ? t[i] : 0.0f);
+                            if (live && v[i]) last[0] = base + js[i] + 1;
+                            continue;
+                        }
                         const float w = __fmul_rn(live ? al[i] : 0.0f, T[0]);
                         c0[0] = fmaf(q5.y, w, c0[0]);
                         c1[0] = fmaf(q5.z, w, c1[0]);
@@ -159,16 +169,14 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                     }
                 }
             }
-            while (P > 1 && m) {
-                const int b = __ffs(m) - 1;
+            while (P > 1 && SPLAT && m) {
+                const int j = w0 + __ffs(m) - 1;
                 m &= m - 1;
-                const int j = w0 + b;
-                typename RecOf<SPLAT>::type r;
-                load_rec(&srec[j * kRF4], r);
-                short4 pr;
-                if (PIXTEST) pr = srect[j];
-                if constexpr (P == 1) {
-                } else if constexpr (SPLAT) {
+                if constexpr (P > 1 && SPLAT) {
+                    SplatRec r;
+                    load_rec(&srec[j * kRF4], r);
+                    short4 pr;
+                    if (PIXTEST) pr = srect[j];
                     SplatCol sc[P / 2];   // pixel columns of the thread
 #pragma unroll
                     for (int c = 0; c < P / 2; ++c) splat_col(r, c ? xf + 1.0f : xf, sc[c]);
@@ -192,38 +200,80 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                         if (valid) last[k] = base + j + 1;
                         if (T[k] < bp.T_stop) live &= ~(1u << k);
                     }
-                } else {   // the same operations, packed over the two rows of a column
+                }
+            }
+            while (P > 1 && !SPLAT && m) {   // the same operations, packed over the two rows of a column
+                if constexpr (P > 1 && !SPLAT) {
+                    constexpr int kN = P == 2 && PIXTEST && !CONE ? 2 : 1, kRow = P / 2;   // pixel k = c + row kRow
+                    int js[kN];
+                    bool in[kN];
+                    float t[kN][P / 2][2];
+                    F2 e2[kN][P / 2];
+                    bool v[kN][P / 2][2];
 #pragma unroll
-                    for (int c = 0; c < P / 2; ++c) {
-                        constexpr int kRow = P / 2;   // pixel k = c + row kRow
-                        ColBase cb;
-                        col_base(r, c ? xf + 1.0f : xf, cb);
-                        float t[2], e[2];
-                        pair_tau2(r, cb, f2_pack(yf, yf + 1.0f), f2_pack(Lp[c], Lp[c + kRow]), t);
+                    for (int i = 0; i < kN; ++i) {
+                        in[i] = m != 0;
+                        js[i] = w0 + (m ? __ffs(m) - 1 : 0);
+                        m &= m - 1;
+                    }
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int k = c + h * kRow;
-                            bool valid = (live >> k) & 1u;
-                            if (PIXTEST) valid = valid && !pixel_outside(x0 + c, y0 + h, pr);
-                            if (COUNT) pairs += valid;
-                            const float t_c = fminf(t[h], bp.tau_max);
-                            valid = valid && t_c >= bp.tau_skip;
-                            t[h] = valid ? t_c : 0.0f;
-                            if (COUNT) blended += valid;
-                            if (valid) last[k] = base + j + 1;
+                    for (int i = 0; i < kN; ++i) {
+                        RecPairs r;
+                        load_rec(&srec[js[i] * kRF4], r);
+                        short4 pr;
+                        if (PIXTEST) pr = srect[js[i]];
+#pragma unroll
+                        for (int c = 0; c < P / 2; ++c) {
+                            ColBase cb;
+                            col_base(r, c ? xf + 1.0f : xf, cb);
+                            float e[2];
+                            pair_tau2(r, cb, f2_pack(yf, yf + 1.0f), f2_pack(Lp[c], Lp[c + kRow]), t[i][c]);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                bool ok = kN == 1 ? ((live >> (c + h * kRow)) & 1u) != 0 : in[i];
+                                if (PIXTEST) ok = ok & !pixel_outside(x0 + c, y0 + h, pr);
+                                if (COUNT) pairs += ok & ((live >> (c + h * kRow)) & 1u);
+                                const float t_c = fminf(t[i][c][h], bp.tau_max);
+                                v[i][c][h] = ok & (t_c >= bp.tau_skip);
+                                t[i][c][h] = v[i][c][h] ? t_c : 0.0f;
+                            }
+                            if (!CONE) {
+                                f2_unpack(f2_mul(f2_dup(-kLog2eF), f2_pack(t[i][c][0], t[i][c][1])), e[0], e[1]);
+                                e2[i][c] = f2_pack(ex2_approx(e[0]), ex2_approx(e[1]));
+                            }
                         }
-                        const F2 tau = f2_pack(t[0], t[1]), Tk = f2_pack(T[c], T[c + kRow]);
-                        f2_unpack(f2_mul(f2_dup(-kLog2eF), tau), e[0], e[1]);
-                        const F2 e2 = f2_pack(ex2_approx(e[0]), ex2_approx(e[1]));
-                        const F2 w = f2_mul(f2_fma(e2, f2_dup(-1.0f), f2_dup(1.0f)), Tk);   // (1 - e2) T
-                        f2_unpack(f2_fma(f2_dup(r.q5.y), w, f2_pack(c0[c], c0[c + kRow])), c0[c], c0[c + kRow]);
-                        f2_unpack(f2_fma(f2_dup(r.q5.z), w, f2_pack(c1[c], c1[c + kRow])), c1[c], c1[c + kRow]);
-                        f2_unpack(f2_fma(f2_dup(r.q5.w), w, f2_pack(c2[c], c2[c + kRow])), c2[c], c2[c + kRow]);
-                        f2_unpack(f2_mul(Tk, e2), T[c], T[c + kRow]);
-                        f2_unpack(f2_add(f2_pack(S[c], S[c + kRow]), tau), S[c], S[c + kRow]);
+                    }
 #pragma unroll
-                        for (int h = 0; h < 2; ++h)
-                            if (T[c + h * kRow] < bp.T_stop) live &= ~(1u << (c + h * kRow));
+                    for (int i = 0; i < kN; ++i) {
+                        const float4 q5 = srec[js[i] * kRF4 + kRF4 - 1];
+#pragma unroll
+                        for (int c = 0; c < P / 2; ++c) {
+                            if (kN > 1 && !CONE) {   // a pixel finished by an earlier record of the batch
+                                float e[2];
+                                f2_unpack(e2[i][c], e[0], e[1]);
+#pragma unroll
+                                for (int h = 0; h < 2; ++h)
+                                    if (!((live >> (c + h * kRow)) & 1u)) e[h] = 1.0f, t[i][c][h] = 0.0f, v[i][c][h] = false;
+                                e2[i][c] = f2_pack(e[0], e[1]);
+                            }
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                if (COUNT) blended += v[i][c][h];
+                                if (v[i][c][h]) last[c + h * kRow] = base + js[i] + 1;
+                            }
+                            f2_unpack(f2_add(f2_pack(S[c], S[c + kRow]), f2_pack(t[i][c][0], t[i][c][1])), S[c], S[c + kRow]);
+                            if constexpr (!CONE) {   // (the projection needs the sum of tau alone)
+                                const F2 Tk = f2_pack(T[c], T[c + kRow]);
+                                const F2 w = f2_mul(f2_fma(e2[i][c], f2_dup(-1.0f), f2_dup(1.0f)), Tk);   // (1 - e2) T
+                                f2_unpack(f2_fma(f2_dup(q5.y), w, f2_pack(c0[c], c0[c + kRow])), c0[c], c0[c + kRow]);
+                                f2_unpack(f2_fma(f2_dup(q5.z), w, f2_pack(c1[c], c1[c + kRow])), c1[c], c1[c + kRow]);
+                                f2_unpack(f2_fma(f2_dup(q5.w), w, f2_pack(c2[c], c2[c + kRow])), c2[c], c2[c + kRow]);
+                                f2_unpack(f2_mul(Tk, e2[i][c]), T[c], T[c + kRow]);
+#pragma unroll
+                                for (int h = 0; h < 2; ++h)
+                                    if (T[c + h * kRow] < bp.T_stop) live &= ~(1u << (c + h * kRow));
+                            }
+                        }
                     }
                 }
             }
@@ -236,6 +286,8 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
         const int x = x0 + L::ox(k), y = y0 + L::oy(k);
         if (x >= V.W || y >= V.H) continue;
         const long long pix = V.pix_base + (long long)y * V.W + x;
+        if constexpr (CONE) T[k] = ex2_approx(__fmul_rn(-kLog2eF, S[k]));
+        if (CONE && l2.weights) l2.weights[pix] = -l2.dproj[pix] * T[k] * exp2f(Lp[k]);
         if (rgb) {   // absent for the cone-beam projection, which needs T alone
             const float o[3] = {fmaf(T[k], bp.bg[0], c0[k]), fmaf(T[k], bp.bg[1], c1[k]), fmaf(T[k], bp.bg[2], c2[k])};
 #pragma unroll
@@ -276,7 +328,7 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
     }
 }
 
-template <int P, bool PIXTEST, bool SPLAT, int CH>
+template <int P, bool PIXTEST, int MODE, int CH>
 static void launch_fwd_ptsc(const ViewInfo *views_d, const int *tile_view, const int *tile_order, long long n_tiles,
                             const uint2 *ranges, const uint32_t *sorted_item, const float4 *rec, const short4 *prect,
                             const BlendParams &bp, float *rgb, float *T_user, float *T_ws, float *S_out,
@@ -286,26 +338,26 @@ static void launch_fwd_ptsc(const ViewInfo *views_d, const int *tile_view, const
     const unsigned threads = (unsigned)(bp.tile_px / P / split);
     n_tiles *= split;
     if (pair_count)
-        pdl_launch(k_render_fwd<P, true, PIXTEST, SPLAT, CH>, (unsigned)n_tiles, threads, 0, st,
+        pdl_launch(k_render_fwd<P, true, PIXTEST, MODE, CH>, (unsigned)n_tiles, threads, 0, st,
             views_d, tile_view, tile_order, ranges, sorted_item, rec, prect, bp, rgb, T_user, T_ws, S_out, nlast_out, tile_replay,
             pair_count, l2, split);
     else
-        pdl_launch(k_render_fwd<P, false, PIXTEST, SPLAT, CH>, (unsigned)n_tiles, threads, 0, st,
+        pdl_launch(k_render_fwd<P, false, PIXTEST, MODE, CH>, (unsigned)n_tiles, threads, 0, st,
             views_d, tile_view, tile_order, ranges, sorted_item, rec, prect, bp, rgb, T_user, T_ws, S_out, nlast_out, tile_replay,
             nullptr, l2, split);
 }
 
-template <int P, bool PIXTEST, bool SPLAT>
+template <int P, bool PIXTEST, int MODE>
 static void launch_fwd_pts(const ViewInfo *views_d, const int *tile_view, const int *tile_order, long long n_tiles,
                            const uint2 *ranges, const uint32_t *sorted_item, const float4 *rec, const short4 *prect,
                            const BlendParams &bp, float *rgb, float *T_user, float *T_ws, float *S_out,
                            uint32_t *nlast_out, uint32_t *tile_replay, unsigned long long *pair_count,
                            const L2Fused &l2, cudaStream_t st) {
     if (bp.chunk_fwd == 64)
-        launch_fwd_ptsc<P, PIXTEST, SPLAT, 64>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect,
+        launch_fwd_ptsc<P, PIXTEST, MODE, 64>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect,
                                                bp, rgb, T_user, T_ws, S_out, nlast_out, tile_replay, pair_count, l2, st);
     else
-        launch_fwd_ptsc<P, PIXTEST, SPLAT, 128>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect,
+        launch_fwd_ptsc<P, PIXTEST, MODE, 128>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect,
                                                 bp, rgb, T_user, T_ws, S_out, nlast_out, tile_replay, pair_count, l2, st);
 }
 
@@ -315,12 +367,19 @@ static void launch_fwd_pt(const ViewInfo *views_d, const int *tile_view, const i
                           const BlendParams &bp, float *rgb, float *T_user, float *T_ws, float *S_out,
                           uint32_t *nlast_out, uint32_t *tile_replay, unsigned long long *pair_count,
                           const L2Fused &l2, cudaStream_t st) {
+    if constexpr (PIXTEST) {   // the projection's tau_skip is 0, below any tau_cut
+        if (!rgb) {
+            launch_fwd_pts<P, PIXTEST, kModeCone>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect,
+                                                  bp, rgb, T_user, T_ws, S_out, nlast_out, tile_replay, pair_count, l2, st);
+            return;
+        }
+    }
     if (bp.splat)
-        launch_fwd_pts<P, PIXTEST, true>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect, bp,
-                                         rgb, T_user, T_ws, S_out, nlast_out, tile_replay, pair_count, l2, st);
+        launch_fwd_pts<P, PIXTEST, kModeSplat>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect, bp,
+                                               rgb, T_user, T_ws, S_out, nlast_out, tile_replay, pair_count, l2, st);
     else
-        launch_fwd_pts<P, PIXTEST, false>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect, bp,
-                                          rgb, T_user, T_ws, S_out, nlast_out, tile_replay, pair_count, l2, st);
+        launch_fwd_pts<P, PIXTEST, kModeBlend>(views_d, tile_view, tile_order, n_tiles, ranges, sorted_item, rec, prect, bp,
+                                               rgb, T_user, T_ws, S_out, nlast_out, tile_replay, pair_count, l2, st);
 }
 
 template <int P>

@@ -209,6 +209,9 @@ struct L2Fused {
     float *grad;
     float *loss;
     float scale;
+    // cone beam (rgb NULL): dL/dproj, and the backward's pixel weights -dL/dproj proj |d_c| (NULL: none)
+    const float *dproj;
+    float *weights;
 };
 
 cudaError_t launch_render_fwd(const ViewInfo *views_d, const int *tile_view, const int *tile_order, long long n_tiles,
@@ -222,6 +225,10 @@ cudaError_t launch_render_bwd(const ViewInfo *views_d, const int *tile_view, con
                               const BlendParams &bp, int ppt, const float *T_fin, const float *S_fin,
                               const uint32_t *nlast, const float *dL_drgb, const float *dL_dT, float *grad_acc,
                               unsigned long long *pair_count, uint32_t *err, cudaStream_t st, long long *launches);
+
+// Cone-beam backward (cone.cu): writes the 16 accumulator values of every item with a footprint.
+cudaError_t launch_cone_bwd(const ViewInfo *views_d, long long n_items, int n_per_view, const float4 *rec,
+                            const short4 *prect, const float *weights, float *acc, cudaStream_t st, long long *launches);
 
 // Longest-first tile order: order[] lists the tiles by descending length (bucketed): the instance
 // count from ranges, or (ranges NULL) the lengths in lens.
