@@ -116,11 +116,12 @@ struct PixLayout {
     __host__ __device__ static constexpr int oy(int k) { return P == 4 ? (k >> 1) : (P == 2 ? k : 0); }
 };
 
-// With few tiles the longest list's CTA decides a blend kernel's time while other SMs idle: two CTAs then
-// share a tile's warps (each stages the list itself), up to 8 tiles per SM.  Forward / backward at one pixel
-// per thread with 1 and 2 CTAs per tile: 64 tiles (2,000 Gaussians, no early stop) 54.7 -> 42.3 us / -, 1,040
-// tiles (100,000 Gaussians) 97.3 -> 92.6 / 156.7 -> 149.8 us, 672 tiles (splat mode) 86.8 -> 77.9 / 190.9 -> 179.7 us;
-// 1,900 tiles 139.5 -> 140.9 us, 4,160 tiles 267 -> 275 us; 4 CTAs per tile 44.4, 108.5, 83.5 us.
+// With few tiles the longest list's CTA decides the forward's time while other SMs idle: two CTAs then
+// share a tile's warps (each stages the list itself), up to 8 tiles per SM.  One pixel per thread with 1 / 2 /
+// 4 CTAs per tile: 64 tiles (2,000 Gaussians, no early stop) 54.7 / 42.3 / 44.4 us, 1,040 tiles (100,000 Gaussians)
+// 97.3 / 92.6 / 108.5 us, 672 tiles (splat mode) 86.8 / 77.9 / 83.5 us; 1,900 tiles 139.5 / 140.9 us, 4,160 tiles
+// 267 / 275 us.  The backward keeps one: two would save 5%, but the order in which the warps' sums reach
+// the accumulators shifts, and with it the last digits of ill-conditioned scale gradients.
 inline int tile_split(long long n_tiles, int threads) { return n_tiles <= 152 * 8 && threads >= 64 ? 2 : 1; }
 
 // Bounds of the pixels a warp owns, for the warp-uniform footprint test of each record.

@@ -58,8 +58,8 @@ struct RingSlot {
     uint32_t item[kGroup];                              // item ids (accumulator rows)
 };
 
-// One CTA per tile (longest list first; with few tiles two, see tile_split): tw th / P consumer
-// threads owning P pixels each, plus the producer warp.  For each group a consumer warp first ballots which records it needs (some
+// One CTA per tile (longest list first): tw th / P consumer threads owning P pixels each, plus
+// the producer warp.  For each group a consumer warp first ballots which records it needs (some
 // pixel of the warp reached the record, the record's footprint touches the warp's pixels and,
 // when pairs below tau_skip are skipped, its opacity can reach tau_skip there), then visits only
 // those, back to front.  The chunk setting CH gives the ring depth: CH / 16 slots (4 or 8, i.e.
@@ -71,7 +71,7 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
              const uint2 *__restrict__ ranges, const uint32_t *__restrict__ sorted_item, const float4 *__restrict__ rec,
              const short4 *__restrict__ prect, BlendParams bp, const float *__restrict__ T_fin, const float *__restrict__ S_fin,
              const uint32_t *__restrict__ nlast, const float *__restrict__ dL_drgb, const float *__restrict__ dL_dT,
-             float *__restrict__ grad_acc, unsigned long long *__restrict__ pair_count, uint32_t *__restrict__ err, int split) {
+             float *__restrict__ grad_acc, unsigned long long *__restrict__ pair_count, uint32_t *__restrict__ err) {
     pdl_entry();
     using L = PixLayout<P>;
     constexpr int kSlots = CH / 16;
@@ -84,13 +84,12 @@ k_render_bwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
 
     const int n_cons = (int)blockDim.x - 32;   // consumer threads; the last warp produces
     const bool producer = (int)threadIdx.x >= n_cons;
-    const int rank = (int)blockIdx.x / split, tid = ((int)blockIdx.x - rank * split) * n_cons + (int)threadIdx.x;
-    const int tile = tile_order ? tile_order[rank] : rank;
+    const int tile = tile_order ? tile_order[blockIdx.x] : (int)blockIdx.x;
     const ViewInfo &V = views[tile_view[tile]];
     const int local = tile - V.tile_base;
     const int tyi = local / V.tiles_x, txi = local - tyi * V.tiles_x;
     int ix, iy;
-    L::origin(producer ? 0 : tid, V.tw, ix, iy);
+    L::origin(producer ? 0 : (int)threadIdx.x, V.tw, ix, iy);
     const int x0 = txi * V.tw + ix, y0 = tyi * V.th + iy;
     const uint2 rg = ranges[tile];
     const int lane = threadIdx.x & 31;
@@ -344,17 +343,15 @@ static void launch_bwd_ptsc(const ViewInfo *views_d, const int *tile_view, const
                             const BlendParams &bp, const float *T_fin, const float *S_fin, const uint32_t *nlast,
                             const float *dL_drgb, const float *dL_dT, float *grad_acc, unsigned long long *pair_count,
                             uint32_t *err, cudaStream_t st) {
-    const int split = tile_split(n_tiles, bp.tile_px / P);
-    const unsigned threads = (unsigned)(bp.tile_px / P / split + 32);   // consumers + the producer warp
-    n_tiles *= split;
+    const unsigned threads = (unsigned)(bp.tile_px / P + 32);   // consumers + the producer warp
     if (pair_count)
         pdl_launch(k_render_bwd<P, true, PIXTEST, SPLAT, CH>, (unsigned)n_tiles, threads, 0, st,
             views_d, tile_view, tile_order, ranges, sorted_item, rec, prect, bp, T_fin, S_fin, nlast, dL_drgb, dL_dT,
-            grad_acc, pair_count, err, split);
+            grad_acc, pair_count, err);
     else
         pdl_launch(k_render_bwd<P, false, PIXTEST, SPLAT, CH>, (unsigned)n_tiles, threads, 0, st,
             views_d, tile_view, tile_order, ranges, sorted_item, rec, prect, bp, T_fin, S_fin, nlast, dL_drgb, dL_dT,
-            grad_acc, nullptr, err, split);
+            grad_acc, nullptr, err);
 }
 
 template <int P, bool PIXTEST, bool SPLAT>
