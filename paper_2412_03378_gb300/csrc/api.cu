@@ -56,7 +56,7 @@ struct vg_workspace {
     DBuf<float> S_fin, T_fin;
     DBuf<uint32_t> nlast;
     DBuf<float> grad;
-    DBuf<uint32_t> hist, scan_tmp;
+    DBuf<uint32_t> hist, hist_tile, scan_tmp;   // scratch of the depth (and other) sorts, the tile sort, the scan
     DBuf<unsigned long long> counters;   // [0] visible items; fwd [1] evaluated, [2] blended pairs; bwd [3], [4];
                                          // [6] instance total of the last scan, [7] look-back timeout flag
     DBuf<float> tomo_cs;
@@ -67,7 +67,8 @@ struct vg_workspace {
     DBuf<float> cone_w;                   // cone-beam backward: pixel weights
     DBuf<float> tomo_dl;                  // tomography backward: dL/dtau of one angle batch's pixels, padded rows
     uint32_t *tile_order = nullptr;       // longest-first tile order of the last bin_sort
-    uint32_t *tile_order_bwd = nullptr;   // longest replay first, from the last forward (NULL: none)
+    bool treplay_clear = false;           // treplay is zero since the last binning
+    bool replay_known = false;            // treplay holds the last forward's replay lengths
     DBuf<uint32_t> treplay, tord_bwd;     // per-tile replay lengths and their order
     int ppt_fwd = 2, ppt_bwd = 1;         // pixels per thread of the blend kernels
     int tuned_fwd = 0, tuned_bwd = 0;     // vg_autotune's choice (0: none yet)
@@ -284,6 +285,7 @@ vg_status vg_workspace_destroy(vg_workspace *ws) {
     release(ws->nlast);
     release(ws->grad);
     release(ws->hist);
+    release(ws->hist_tile);
     release(ws->scan_tmp);
     release(ws->counters);
     release(ws->tomo_cs);
@@ -328,8 +330,13 @@ static vg_status reserve_sort_scratch(vg_workspace *ws, long long n) {
 
 static unsigned long long *total64_ptr(vg_workspace *ws) { return ws->counters.p + 6; }
 static uint32_t *lookback_err_ptr(vg_workspace *ws) { return (uint32_t *)(ws->counters.p + 7); }
-// The backward's tile order: by the replay lengths the last forward measured, else the binning's.
-static const uint32_t *bwd_order(vg_workspace *ws) { return ws->tile_order_bwd ? ws->tile_order_bwd : ws->tile_order; }
+// The backward's tile order: by the replay lengths the last forward measured (longest first), else the binning's.
+static cudaError_t bwd_order(vg_workspace *ws, cudaStream_t st, const int **order) {
+    *order = (const int *)ws->tile_order;
+    if (!ws->replay_known) return cudaSuccess;
+    *order = (const int *)ws->tord_bwd.p;
+    return launch_tile_order(nullptr, ws->treplay.p, ws->n_tiles, ws->tord_bwd.p, st, &ws->launches);
+}
 
 // Reports (and clears) error bits latched on the device: a look-back timeout, a capacity
 // overflow.  Reads h_total[2] as filled by the last copy of counters[6..7].
@@ -388,6 +395,7 @@ vg_status vg_workspace_reserve(vg_workspace *ws, int64_t n_items, int64_t n_inst
     vg_status s = reserve_items(ws, n_items);
     if (s == VG_OK) s = reserve_sort_scratch(ws, n_items);
     if (s == VG_OK) s = reserve_instances(ws, n_instances);
+    if (s == VG_OK) s = ensure(ws, ws->hist_tile, radix_scratch_words(ws->capacity, 32), "radix sort scratch");
     if (s == VG_OK) s = ensure(ws, ws->S_fin, (size_t)n_pixels, "pixel state");
     if (s == VG_OK) s = ensure(ws, ws->T_fin, (size_t)n_pixels, "pixel state");
     if (s == VG_OK) s = ensure(ws, ws->nlast, (size_t)n_pixels, "pixel state");
@@ -574,21 +582,46 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
     // binning ahead of the count's readback on instance buffers left by an earlier call (below);
     // the sort scratch for both sorts is reserved before anything is enqueued
     const bool ahead = !fixed && ws->capacity > 0 && ws->ikey[1].p != nullptr;
-    VG_TRY(reserve_sort_scratch(ws, ahead ? std::max(n, ws->capacity) : n));
+    const bool small = n >= 1 && n <= kSmallItems, known = ahead || (fixed && ws->capacity > 0);
+    VG_TRY(reserve_sort_scratch(ws, n));
+    VG_TRY(ensure(ws, ws->ranges, (size_t)ws->n_tiles, "tile ranges"));
+    VG_TRY(ensure(ws, ws->tord, (size_t)ws->n_tiles, "tile order"));
+    // the tile sort's scratch: its own where the capacity is known and it may be had, so that it is cleared in advance
+    const size_t tile_words = known ? radix_scratch_words(ws->capacity, 32) : 0;
+    const bool own = known && (ws->hist_tile.n >= tile_words || !fixed || !ws->hist_tile.p);
+    if (own) VG_TRY(ensure(ws, ws->hist_tile, tile_words, "radix sort scratch"));
     // 1. items by depth key (stable: ties keep index order)
     {
         ProfScope ps(ws, ST_DEPTH, st);
-        uint32_t *ksorted = nullptr;
-        VG_CUDA(ws, launch_radix_sort(ws->depth.p, nullptr, ws->skey[0].p, ws->sval[0].p, ws->skey[1].p,
-                                      ws->sval[1].p, n, nullptr, 32, ws->hist.p, lookback_err_ptr(ws), &ksorted,
-                                      &ws->perm, st, &ws->launches));
+        // what the binning and the forward want zeroed, in one launch (the replay lengths where a forward has made
+        // their buffer large enough)
+        ClearList cl;
+        if (!small && n > 0) cl.add(ws->hist.p, radix_scratch_words(n, 32));
+        if (!small) cl.add(ws->scan_tmp.p, scan_tmp_words(n));
+        if (own) cl.add(ws->hist_tile.p, radix_scratch_words(ws->capacity, bits_for(ws->n_tiles)));
+        cl.add(reinterpret_cast<uint32_t *>(ws->ranges.p), 2 * (size_t)ws->n_tiles);
+        ws->treplay_clear = ws->treplay.p && ws->treplay.n >= (size_t)ws->n_tiles;
+        if (ws->treplay_clear) cl.add(ws->treplay.p, (size_t)ws->n_tiles);
+        VG_CUDA(ws, launch_clear(cl, st, &ws->launches));
+        if (small) {   // with the offsets of step 2
+            ws->perm = ws->sval[1].p;
+            VG_CUDA(ws, launch_small_order(ws->depth.p, ws->count.p, (int)n, ws->perm, ws->offsets.p, total64_ptr(ws),
+                                           fixed ? (unsigned long long)ws->capacity : ~0ull, lookback_err_ptr(ws), st,
+                                           &ws->launches));
+        } else {
+            uint32_t *ksorted = nullptr;
+            VG_CUDA(ws, launch_radix_sort(ws->depth.p, nullptr, ws->skey[0].p, ws->sval[0].p, ws->skey[1].p,
+                                          ws->sval[1].p, n, nullptr, 32, ws->hist.p, lookback_err_ptr(ws), true,
+                                          &ksorted, &ws->perm, st, &ws->launches));
+        }
     }
     // 2. instance offsets in depth order
     {
         ProfScope ps(ws, ST_SCAN, st);
-        VG_CUDA(ws, launch_scan_gather(ws->count.p, ws->perm, ws->offsets.p, n, ws->scan_tmp.p, total64_ptr(ws),
-                                       fixed ? (unsigned long long)ws->capacity : ~0ull, lookback_err_ptr(ws), st,
-                                       &ws->launches));
+        if (!small)
+            VG_CUDA(ws, launch_scan_gather(ws->count.p, ws->perm, ws->offsets.p, n, ws->scan_tmp.p, total64_ptr(ws),
+                                           fixed ? (unsigned long long)ws->capacity : ~0ull, lookback_err_ptr(ws), true,
+                                           st, &ws->launches));
     }
     // The instance count: read back (one synchronisation), or, with a fixed capacity, left on
     // the device; the kernels below then cover the capacity and read the count themselves.
@@ -596,7 +629,8 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
     // binning is enqueued on them first in the same device-count form (kernels stop at the
     // capacity) and the count is read back afterwards, so the GPU keeps working through the
     // readback; a step with more instances than the buffers hold is binned again after they grow.
-    auto bin_rest = [&](long long total, const unsigned long long *total_dev) -> vg_status {
+    bool ranges_clear = true;
+    auto bin_rest = [&](long long total, const unsigned long long *total_dev, bool cleared) -> vg_status {   // cleared: hist_tile
         // 3. duplicate in depth order, 4. stable sort by tile id, 5. per-tile ranges
         {
             ProfScope ps(ws, ST_DUP, st);
@@ -606,17 +640,16 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
         {
             ProfScope ps(ws, ST_TILE, st);
             VG_CUDA(ws, launch_radix_sort(ws->ikey[0].p, ws->ival[0].p, ws->ikey[1].p, ws->ival[1].p, ws->ikey[0].p,
-                                          ws->ival[0].p, total, total_dev, bits_for(ws->n_tiles), ws->hist.p,
-                                          lookback_err_ptr(ws), &ws->inst_key, &ws->inst_item, st, &ws->launches));
+                                          ws->ival[0].p, total, total_dev, bits_for(ws->n_tiles),
+                                          cleared ? ws->hist_tile.p : ws->hist.p, lookback_err_ptr(ws), cleared, &ws->inst_key, &ws->inst_item, st, &ws->launches));
         }
-        VG_TRY(ensure(ws, ws->ranges, (size_t)ws->n_tiles, "tile ranges"));
-        VG_TRY(ensure(ws, ws->tord, (size_t)ws->n_tiles, "tile order"));
         {
             ProfScope ps(ws, ST_RANGES, st);
-            VG_CUDA(ws, launch_ranges(ws->inst_key, total, total_dev, ws->ranges.p, ws->n_tiles, st, &ws->launches));
+            VG_CUDA(ws, launch_ranges(ws->inst_key, total, total_dev, ws->ranges.p, ws->n_tiles, ranges_clear, st, &ws->launches));
             VG_CUDA(ws, launch_tile_order(ws->ranges.p, nullptr, ws->n_tiles, ws->tord.p, st, &ws->launches));
             ws->tile_order = ws->tord.p;
-            ws->tile_order_bwd = nullptr;   // until a forward has measured the replay lengths
+            ws->replay_known = false;   // until a forward has measured the replay lengths
+            ranges_clear = false;       // a binning again after the buffers have grown clears them itself
         }
         return VG_OK;
     };
@@ -624,12 +657,12 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
         if (ws->capacity <= 0 || !ws->ikey[1].p)
             return fail(ws, VG_ERR_CAPACITY, "fixed capacity: reserve instances with vg_workspace_reserve first");
         ws->n_inst = -1;   // known on the device only
-        VG_TRY(bin_rest(ws->capacity, total64_ptr(ws)));
+        VG_TRY(bin_rest(ws->capacity, total64_ptr(ws), own));
     } else {
         long long total;
         if (ahead) {
             VG_TRY(read_total_start(ws, st));
-            VG_TRY(bin_rest(ws->capacity, total64_ptr(ws)));
+            VG_TRY(bin_rest(ws->capacity, total64_ptr(ws), own));
             VG_TRY(read_total_finish(ws, st, &total));
         } else {
             VG_TRY(read_total(ws, st, &total));
@@ -640,7 +673,7 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
             // the binning enqueued ahead still uses the buffers about to be replaced
             if (ahead) VG_CUDA(ws, cudaStreamSynchronize(st));
             VG_TRY(reserve_instances(ws, total));
-            VG_TRY(bin_rest(total, nullptr));
+            VG_TRY(bin_rest(total, nullptr, false));
         }
         ws->n_inst = total;
     }
@@ -667,13 +700,12 @@ static vg_status render_fwd_impl(vg_workspace *ws, float *rgb, float *T_final, v
     VG_TRY(ensure(ws, ws->tord_bwd, (size_t)std::max<long long>(ws->n_tiles, 1), "backward tile order"));
     {
         ProfScope ps(ws, ST_FWD, st);
-        VG_CUDA(ws, cudaMemsetAsync(ws->treplay.p, 0, sizeof(uint32_t) * (size_t)ws->n_tiles, st));
+        if (!ws->treplay_clear) VG_CUDA(ws, cudaMemsetAsync(ws->treplay.p, 0, sizeof(uint32_t) * (size_t)ws->n_tiles, st));
+        ws->treplay_clear = false;
         VG_CUDA(ws, launch_render_fwd(ws->views.p, ws->tile_view.p, (const int *)ws->tile_order, ws->n_tiles,
                                       ws->ranges.p, ws->inst_item, ws->rec.p, ws->prect.p, ws->bp, ws->ppt_fwd, rgb, T_final,
                                       ws->T_fin.p, ws->S_fin.p, ws->nlast.p, ws->treplay.p, pc, l2, st, &ws->launches));
-        // the backward's order: longest replay (largest last blended position in the tile) first
-        VG_CUDA(ws, launch_tile_order(nullptr, ws->treplay.p, ws->n_tiles, ws->tord_bwd.p, st, &ws->launches));
-        ws->tile_order_bwd = ws->tord_bwd.p;
+        ws->replay_known = true;
     }
     ws->stage = 3;
     return VG_OK;
@@ -718,12 +750,14 @@ static vg_status render_bwd_impl(vg_workspace *ws, const float *dL_drgb, const f
         if (cone_weights)
             VG_CUDA(ws, launch_cone_bwd(ws->views.p, ws->n_items, ws->g.n, ws->rec.p, ws->prect.p, cone_weights, ws->grad.p,
                                         st, &ws->launches));
-        else
-            VG_CUDA(ws, launch_render_bwd(ws->views.p, ws->tile_view.p, (const int *)bwd_order(ws), ws->n_tiles,
-                                      ws->ranges.p, ws->inst_item, ws->rec.p, ws->prect.p, ws->bp, ws->ppt_bwd,
-                                      ws->T_fin.p,
-                                      ws->S_fin.p, ws->nlast.p, dL_drgb, dL_dT, ws->grad.p, pc, lookback_err_ptr(ws),
-                                      st, &ws->launches));
+        else {
+            const int *order;
+            VG_CUDA(ws, bwd_order(ws, st, &order));
+            VG_CUDA(ws, launch_render_bwd(ws->views.p, ws->tile_view.p, order, ws->n_tiles, ws->ranges.p, ws->inst_item,
+                                          ws->rec.p, ws->prect.p, ws->bp, ws->ppt_bwd, ws->T_fin.p, ws->S_fin.p,
+                                          ws->nlast.p, dL_drgb, dL_dT, ws->grad.p, pc, lookback_err_ptr(ws), st,
+                                          &ws->launches));
+        }
     }
     {
         // the chain writes every Gaussian's gradient: overwriting with VG_FLAG_GRAD_ZERO, else adding
@@ -863,7 +897,7 @@ vg_status vg_query_density(vg_workspace *ws, const vg_gaussians *g, const vg_gri
     {
         ProfScope ps(ws, ST_SCAN, st);
         VG_CUDA(ws, launch_scan_gather(ws->count.p, nullptr, ws->offsets.p, n, ws->scan_tmp.p, total64_ptr(ws), ~0ull,
-                                       lookback_err_ptr(ws), st, &ws->launches));
+                                       lookback_err_ptr(ws), false, st, &ws->launches));
     }
     long long total = 0;
     VG_TRY(read_total(ws, st, &total));
@@ -881,11 +915,11 @@ vg_status vg_query_density(vg_workspace *ws, const vg_gaussians *g, const vg_gri
         ProfScope ps(ws, ST_TILE, st);
         VG_CUDA(ws, launch_radix_sort(ws->ikey[0].p, ws->ival[0].p, ws->ikey[1].p, ws->ival[1].p, ws->ikey[0].p,
                                       ws->ival[0].p, total, nullptr, bits_for(bricks), ws->hist.p,
-                                      lookback_err_ptr(ws), &keys, &vals, st, &ws->launches));
+                                      lookback_err_ptr(ws), false, &keys, &vals, st, &ws->launches));
     }
     {
         ProfScope ps(ws, ST_RANGES, st);
-        VG_CUDA(ws, launch_ranges(keys, total, nullptr, ws->ranges.p, bricks, st, &ws->launches));
+        VG_CUDA(ws, launch_ranges(keys, total, nullptr, ws->ranges.p, bricks, false, st, &ws->launches));
     }
     {
         ProfScope ps(ws, ST_VOXEL, st);
@@ -937,7 +971,9 @@ vg_status vg_render_bwd_noalloc(vg_workspace *ws, const float *dL_drgb, const fl
     }
     {
         ProfScope ps(ws, ST_BWD, st);
-        VG_CUDA(ws, launch_render_bwd(ws->views.p, ws->tile_view.p, (const int *)bwd_order(ws), ws->n_tiles,
+        const int *order;
+        VG_CUDA(ws, bwd_order(ws, st, &order));
+        VG_CUDA(ws, launch_render_bwd(ws->views.p, ws->tile_view.p, order, ws->n_tiles,
                                       ws->ranges.p, ws->inst_item, ws->rec.p, ws->prect.p, ws->bp, ws->ppt_bwd,
                                       ws->T_fin.p, ws->S_fin.p, ws->nlast.p, dL_drgb, dL_dT, acc, pc,
                                       lookback_err_ptr(ws), st, &ws->launches));
@@ -1095,7 +1131,7 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
         {
             ProfScope ps(ws, ST_SCAN, st);
             VG_CUDA(ws, launch_scan_gather(ws->count.p, nullptr, ws->offsets.p, items, ws->scan_tmp.p,
-                                           total64_ptr(ws), ~0ull, lookback_err_ptr(ws), st, &ws->launches));
+                                           total64_ptr(ws), ~0ull, lookback_err_ptr(ws), false, st, &ws->launches));
         }
         long long total = 0;
         VG_TRY(read_total(ws, st, &total));
@@ -1111,12 +1147,12 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
             ProfScope ps(ws, ST_TILE, st);
             VG_CUDA(ws, launch_radix_sort(ws->ikey[0].p, ws->ival[0].p, ws->ikey[1].p, ws->ival[1].p, ws->ikey[0].p,
                                           ws->ival[0].p, total, nullptr, bits_for(n_tiles), ws->hist.p,
-                                          lookback_err_ptr(ws), &ws->inst_key, &ws->inst_item, st, &ws->launches));
+                                          lookback_err_ptr(ws), false, &ws->inst_key, &ws->inst_item, st, &ws->launches));
         }
         VG_TRY(ensure(ws, ws->ranges, (size_t)n_tiles, "tile ranges"));
         {
             ProfScope ps(ws, ST_RANGES, st);
-            VG_CUDA(ws, launch_ranges(ws->inst_key, total, nullptr, ws->ranges.p, n_tiles, st, &ws->launches));
+            VG_CUDA(ws, launch_ranges(ws->inst_key, total, nullptr, ws->ranges.p, n_tiles, false, st, &ws->launches));
         }
         float *proj_b = proj + (size_t)a0 * det_px;
         if (!proj_given) {
@@ -1137,7 +1173,7 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
             ProfScope ps(ws, ST_TBWD, st);
             if (by_home)
                 VG_CUDA(ws, launch_radix_sort(home, nullptr, ws->skey[1].p, ws->sval[1].p, ws->skey[0].p, ws->sval[0].p, items,
-                                              nullptr, bits_for(n_tiles + 1), ws->hist.p, lookback_err_ptr(ws), &home, &order, st,
+                                              nullptr, bits_for(n_tiles + 1), ws->hist.p, lookback_err_ptr(ws), false, &home, &order, st,
                                               &ws->launches));
             VG_CUDA(ws, launch_tomo_bwd(items, N, beam->det_w, beam->det_h, order, ws->count.p, ws->rec.p, ws->tomo_dl.p,
                                         ws->grad.p, st, &ws->launches));
@@ -1327,7 +1363,7 @@ vg_status vg_query(vg_workspace *ws, vg_stats *out, void *stream) {
     out->launches = ws->launches;
     size_t bytes = ws->views.n * sizeof(ViewInfo) + ws->tile_view.n * 4 + ws->rec.n * 16 + ws->depth.n * 4 +
                    ws->count.n * 4 + ws->offsets.n * 4 + ws->rect.n * 8 + ws->ranges.n * 8 + ws->S_fin.n * 4 +
-                   ws->T_fin.n * 4 + ws->nlast.n * 4 + ws->grad.n * 4 + ws->hist.n * 4 + ws->scan_tmp.n * 4;
+                   ws->T_fin.n * 4 + ws->nlast.n * 4 + ws->grad.n * 4 + (ws->hist.n + ws->hist_tile.n) * 4 + ws->scan_tmp.n * 4;
     for (int k = 0; k < 2; ++k)
         bytes += (ws->skey[k].n + ws->sval[k].n + ws->ikey[k].n + ws->ival[k].n) * 4;
     out->device_bytes = (int64_t)bytes;

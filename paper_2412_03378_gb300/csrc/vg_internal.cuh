@@ -161,16 +161,35 @@ cudaError_t launch_tomo_preprocess(const GaussIn &g, const float *cs_d /* [A][2]
                                    float tau_cut, float4 *rec, uint32_t *count, short4 *rect, uint32_t *home,
                                    cudaStream_t st, long long *launches);
 
+// Buffers (16-byte aligned, in 32-bit words) zeroed by one launch.
+struct ClearList {
+    static constexpr int kMax = 5;
+    uint32_t *p[kMax] = {};
+    size_t words[kMax] = {};
+    int n = 0;
+    void add(uint32_t *q, size_t w) { p[n] = q, words[n++] = w; }
+};
+cudaError_t launch_clear(const ClearList &c, cudaStream_t st, long long *launches);
+
 // Error bits latched in the workspace's device flag word.
 constexpr uint32_t kDevErrTimeout = 1u, kDevErrCapacity = 2u;
 
+// `cleared` below: the caller has zeroed the scratch (or ranges) already, else the launcher does.
+//
 // Single-pass exclusive scan of count[perm[i]] (perm may be NULL) into out[0..n); out[n] and
 // *total64 receive the total.  tmp must hold scan_tmp_words(n) uint32; *err gets
 // kDevErrTimeout if a look-back wait timed out and kDevErrCapacity if the total exceeds cap.
 size_t scan_tmp_words(long long n);
 cudaError_t launch_scan_gather(const uint32_t *count, const uint32_t *perm, uint32_t *out, long long n,
                                uint32_t *tmp, unsigned long long *total64, unsigned long long cap, uint32_t *err,
-                               cudaStream_t st, long long *launches);
+                               bool cleared, cudaStream_t st, long long *launches);
+
+// Depth order and instance offsets of 1 .. kSmallItems items by one CTA: perm lists the items by key
+// (stable), offsets, total64 and *err as the scan above leaves them.
+constexpr int kSmallItems = 4096;
+cudaError_t launch_small_order(const uint32_t *keys, const uint32_t *count, int n, uint32_t *perm, uint32_t *offsets,
+                               unsigned long long *total64, unsigned long long cap, uint32_t *err, cudaStream_t st,
+                               long long *launches);
 
 // Stable LSD radix sort of (key, value) pairs over key bits [0, bits) (n < 2^30), one kernel
 // per 8-bit digit.  Reads keys_in / vals_in (vals_in NULL: values are the input positions);
@@ -181,8 +200,8 @@ cudaError_t launch_scan_gather(const uint32_t *count, const uint32_t *perm, uint
 size_t radix_scratch_words(long long n, int bits);
 cudaError_t launch_radix_sort(const uint32_t *keys_in, const uint32_t *vals_in, uint32_t *ka, uint32_t *va,
                               uint32_t *kb, uint32_t *vb, long long n, const unsigned long long *n_dev, int bits,
-                              uint32_t *scratch, uint32_t *err, uint32_t **keys_out, uint32_t **vals_out,
-                              cudaStream_t st, long long *launches);
+                              uint32_t *scratch, uint32_t *err, bool cleared, uint32_t **keys_out,
+                              uint32_t **vals_out, cudaStream_t st, long long *launches);
 
 // A look-back over a status array (4 zero words, device) whose predecessor never publishes, with a
 // spin limit of spin_limit polls; the wait gives up and sets kDevErrTimeout in *err (test path).
@@ -200,7 +219,7 @@ cudaError_t launch_duplicate(const uint32_t *perm, const uint32_t *offsets, cons
                              uint32_t *inst_val, long long capacity, cudaStream_t st, long long *launches);
 
 cudaError_t launch_ranges(const uint32_t *sorted_key, long long n_inst, const unsigned long long *n_dev, uint2 *ranges,
-                          long long n_tiles, cudaStream_t st, long long *launches);
+                          long long n_tiles, bool cleared, cudaStream_t st, long long *launches);
 
 // The L2 image loss fused into the forward's epilogue (target NULL: none): *loss +=
 // scale sum (rgb - target)^2 and grad = 2 scale (rgb - target), per pixel where rgb is written.
