@@ -150,6 +150,9 @@ typedef struct {
 #define VG_FLAG_PROJ_GIVEN 32u     /* vg_project_tomo with dL_dproj: proj already holds the
                                       projection of the same Gaussians, beam and options (from an
                                       earlier call), so it is not recomputed before the backward */
+#define VG_FLAG_NO_LISTS 64u       /* with VG_FLAG_PROJ_GIVEN: the tile lists, which the gradient
+                                      does not use, are not formed; the list read-backs keep what
+                                      the workspace's last tomography call with lists left */
 #define VG_FLAG_SPLAT 16u          /* the 3DGS comparison mode (Sec. 3.2, Eq. 5-7) in the same
                                       pipeline: the density input holds the peak opacity o and
                                       alpha = min(o G'(p), alpha_max), G' the 2D Gaussian with
@@ -256,6 +259,11 @@ vg_status vg_render_fwd_l2(vg_workspace *ws, float *rgb, float *T_final, const f
 vg_status vg_render_bwd(vg_workspace *ws, const float *dL_drgb, const float *dL_dT,
                         float *dmu, float *dscale, float *dquat, float *dkappa, float *dsh,
                         void *stream);
+
+/* vg_render_bwd writing every gradient (as with VG_FLAG_GRAD_ZERO), whatever the options of the
+ * last vg_preprocess: buffers need not be initialised. */
+vg_status vg_render_bwd_set(vg_workspace *ws, const float *dL_drgb, const float *dL_dT, float *dmu, float *dscale,
+                            float *dquat, float *dkappa, float *dsh, void *stream);
 
 /* Backward that allocates no device memory.  The paper has no counterpart: this is a
  * library-usage variant of vg_render_bwd with the same arguments and results.

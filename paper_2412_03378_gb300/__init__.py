@@ -8,6 +8,7 @@ PyTorch fallback: if the library is missing, `load()` raises.
 """
 from __future__ import annotations
 
+import copy
 import ctypes
 import math
 import os
@@ -27,6 +28,7 @@ FLAG_GRAD_ZERO = 4
 FLAG_DENSITY_THETA = 8
 FLAG_SPLAT = 16
 FLAG_PROJ_GIVEN = 32
+FLAG_NO_LISTS = 64
 # stage names of the event profiler, in the bit order of vg_profile_stages
 STAGES = ("preprocess", "depth_sort", "scan", "duplicate", "tile_sort", "ranges", "render_fwd", "render_bwd",
           "chain", "l2_loss", "tomo_fwd", "tomo_bwd", "voxel_eval", "ray_march")
@@ -99,6 +101,7 @@ _SIGS = {
     "vg_render_fwd_l2": [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_float,
                          ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p],
     "vg_render_bwd": [ctypes.c_void_p] + [ctypes.c_void_p] * 7 + [ctypes.c_void_p],
+    "vg_render_bwd_set": [ctypes.c_void_p] + [ctypes.c_void_p] * 7 + [ctypes.c_void_p],
     "vg_render_bwd_noalloc": [ctypes.c_void_p] + [ctypes.c_void_p] * 7 + [ctypes.c_void_p],
     "vg_project_tomo": [ctypes.c_void_p] * 11,
     "vg_project_cone": [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32] + [ctypes.c_void_p] * 8,
@@ -146,8 +149,10 @@ def _ptr(t):
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    # the raw handle: building a torch.cuda.Stream object for each library call costs several times as much
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 _DT = {torch.float32: VG_F32, torch.bfloat16: VG_BF16, torch.float16: VG_F16}
@@ -233,11 +238,8 @@ class Gaussians:
 def camera_struct(cam):
     """Any object with R (3x3), t (3), fx, fy, cx, cy, width, height."""
     c = _Camera()
-    R = [float(x) for row in cam.R for x in row]
-    for k in range(9):
-        c.R[k] = R[k]
-    for k in range(3):
-        c.t[k] = float(cam.t[k])
+    c.R[:] = [float(x) for row in cam.R for x in row]
+    c.t[:] = [float(x) for x in cam.t]
     c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
     c.width, c.height = int(cam.width), int(cam.height)
     return c
@@ -310,6 +312,11 @@ class Workspace:
         self._chk(self._L.vg_render_bwd(self.h, _ptr(dL_drgb), _ptr(dL_dT), _ptr(dmu), _ptr(dscale), _ptr(dquat),
                                         _ptr(dkappa), _ptr(dsh), _stream(stream)))
 
+    def render_bwd_set(self, dL_drgb, dL_dT, dmu, dscale, dquat, dkappa, dsh, stream=None):
+        """vg_render_bwd_set: the backward writing every gradient, whatever the buffers hold."""
+        self._chk(self._L.vg_render_bwd_set(self.h, _ptr(dL_drgb), _ptr(dL_dT), _ptr(dmu), _ptr(dscale), _ptr(dquat),
+                                            _ptr(dkappa), _ptr(dsh), _stream(stream)))
+
     def render_bwd_noalloc(self, dL_drgb, dL_dT, dmu, dscale, dquat, dkappa, dsh, stream=None):
         """vg_render_bwd_noalloc: the backward without any device allocation (see vg.h)."""
         self._chk(self._L.vg_render_bwd_noalloc(self.h, _ptr(dL_drgb), _ptr(dL_dT), _ptr(dmu), _ptr(dscale),
@@ -336,6 +343,7 @@ class Workspace:
         b.det_w, b.det_h = int(beam.det_w), int(beam.det_h)
         b.pitch_u, b.pitch_v, b.u0, b.v0 = float(beam.pitch_u), float(beam.pitch_v), float(beam.u0), float(beam.v0)
         oc = opts.c()
+        self.generation += 1
         self._chk(self._L.vg_project_tomo(self.h, ctypes.byref(g.c()), ctypes.byref(b), ctypes.byref(oc), _ptr(proj),
                                           _ptr(dL_dproj), _ptr(dmu), _ptr(dscale), _ptr(dquat), _ptr(dkappa),
                                           _stream(stream)))
@@ -349,6 +357,7 @@ class Workspace:
         b.det_w, b.det_h = int(beam.det_w), int(beam.det_h)
         b.pitch_u, b.pitch_v, b.u0, b.v0 = float(beam.pitch_u), float(beam.pitch_v), float(beam.u0), float(beam.v0)
         oc = opts.c()
+        self.generation += 1
         self._chk(self._L.vg_tomo_l2_step(self.h, ctypes.byref(g.c()), ctypes.byref(b), ctypes.byref(oc), _ptr(target),
                                           float(scale), _ptr(proj), _ptr(loss), _ptr(dmu), _ptr(dscale), _ptr(dquat),
                                           _ptr(dkappa), _stream(stream)))
@@ -370,6 +379,7 @@ class Workspace:
             gr.origin[a], gr.voxel[a] = float(origin[a]), float(voxel[a])
         gr.nx, gr.ny, gr.nz = (int(d) for d in dims)
         oc = opts.c()
+        self.generation += 1
         self._chk(self._L.vg_query_density(self.h, ctypes.byref(g.c()), ctypes.byref(gr), ctypes.byref(oc), _ptr(out),
                                            _stream(stream)))
 
@@ -459,6 +469,7 @@ class _RenderFn(torch.autograd.Function):
         ws.bin_sort()
         ws.render_fwd(rgb, T)
         ctx.ws, ctx.gen, ctx.g = ws, ws.generation, g
+        ctx.set_materialize_grads(False)   # an output the loss does not use costs nothing
         return rgb, T
 
     @staticmethod
@@ -466,21 +477,19 @@ class _RenderFn(torch.autograd.Function):
         ws, g = ctx.ws, ctx.g
         if ws.generation != ctx.gen:
             raise RuntimeError("the workspace was reused by another forward before this backward")
-        dmu = torch.zeros_like(g.mu, dtype=torch.float32)
-        dscale = torch.zeros_like(g.scale, dtype=torch.float32)
-        dquat = torch.zeros_like(g.quat, dtype=torch.float32)
-        dkappa = torch.zeros_like(g.kappa, dtype=torch.float32)
-        dsh = torch.zeros_like(g.sh, dtype=torch.float32)
+        dmu, dscale, dquat, dkappa, dsh = (torch.empty_like(t, dtype=torch.float32)
+                                           for t in (g.mu, g.scale, g.quat, g.kappa, g.sh))
         g_rgb = (g_rgb if g_rgb is not None else torch.zeros((n_pixels_ws(ws), 3), device=g.mu.device)).contiguous()
         g_T = g_T.contiguous() if g_T is not None else None
-        ws.render_bwd(g_rgb.float(), None if g_T is None else g_T.float(), dmu, dscale, dquat, dkappa, dsh)
+        ws.render_bwd_set(g_rgb.float(), None if g_T is None else g_T.float(), dmu, dscale, dquat, dkappa, dsh)
         return (None, None, None, None, dmu.to(g.mu.dtype), dscale.to(g.scale.dtype), dquat.to(g.quat.dtype),
                 dkappa.to(g.kappa.dtype), dsh.to(g.sh.dtype))
 
 
 class _TomoFn(torch.autograd.Function):
-    """proj = exp(-sum tau) of a parallel beam (vg_project_tomo); the backward calls it again
-    with dL/dproj, which recomputes the projection and accumulates the gradients."""
+    """proj = exp(-sum tau) of a parallel beam (vg_project_tomo); the backward calls it again with
+    dL/dproj.  It hands over its own copy of the projection, and leaves the workspace's tile lists
+    alone while they are the forward's; parameters written to in between are projected anew."""
 
     @staticmethod
     def forward(ctx, ws, beam, opts, mu, scale, quat, kappa):
@@ -489,16 +498,36 @@ class _TomoFn(torch.autograd.Function):
         proj = torch.empty((len(beam.angles), int(beam.det_h), int(beam.det_w)), device=mu.device,
                            dtype=torch.float32)
         ws.project_tomo(g, beam, opts, proj)
-        ctx.ws, ctx.beam, ctx.opts, ctx.g = ws, beam, opts, g
+        ctx.ws, ctx.beam, ctx.opts, ctx.g, ctx.gen = ws, beam, opts, g, ws.generation
+        ctx.seen = [t._version for t in (g.mu, g.scale, g.quat, g.kappa)]
+        ctx.angles = [float(a) for a in beam.angles]
+        ctx.geometry = (int(beam.det_w), int(beam.det_h), float(beam.pitch_u), float(beam.pitch_v), float(beam.u0),
+                        float(beam.v0), opts.tau_cut, opts.flags)
+        try:
+            ctx.proj = proj.clone()
+        except torch.OutOfMemoryError:
+            ctx.proj = None
         return proj
 
     @staticmethod
     def backward(ctx, g_proj):
-        g = ctx.g
-        grads = [torch.zeros_like(t, dtype=torch.float32) for t in (g.mu, g.scale, g.quat, g.kappa)]
-        proj = torch.empty_like(g_proj, dtype=torch.float32)
-        ctx.ws.project_tomo(g, ctx.beam, ctx.opts, proj, g_proj.contiguous().float(), *grads)
-        return (None, None, None) + tuple(d.to(t.dtype) for d, t in zip(grads, (g.mu, g.scale, g.quat, g.kappa)))
+        g, beam, opts = ctx.g, ctx.beam, ctx.opts
+        params = (g.mu, g.scale, g.quat, g.kappa)
+        grads = [torch.empty_like(t, dtype=torch.float32) for t in params]
+        flags = opts.flags | FLAG_GRAD_ZERO
+        same = ctx.proj is not None and ctx.seen == [t._version for t in params] and \
+            ctx.geometry == (int(beam.det_w), int(beam.det_h), float(beam.pitch_u), float(beam.pitch_v), float(beam.u0),
+                             float(beam.v0), opts.tau_cut, opts.flags) and \
+            ctx.angles == [float(a) for a in beam.angles]
+        if same:
+            proj = ctx.proj
+            flags |= FLAG_PROJ_GIVEN | (FLAG_NO_LISTS if ctx.ws.generation == ctx.gen else 0)
+        else:
+            proj = torch.empty_like(g_proj, dtype=torch.float32)
+        o = copy.copy(opts)
+        o.flags = flags
+        ctx.ws.project_tomo(g, beam, o, proj, g_proj.contiguous().float(), *grads)
+        return (None, None, None) + tuple(d.to(t.dtype) for d, t in zip(grads, params))
 
 
 class _ConeFn(torch.autograd.Function):

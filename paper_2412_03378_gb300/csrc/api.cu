@@ -729,7 +729,7 @@ vg_status vg_render_fwd_l2(vg_workspace *ws, float *rgb, float *T_final, const f
 
 static vg_status render_bwd_impl(vg_workspace *ws, const float *dL_drgb, const float *dL_dT, float *dmu, float *dscale,
                                  float *dquat, float *dkappa, float *dsh, void *stream, bool drgb_optional,
-                                 const float *cone_weights = nullptr) {
+                                 const float *cone_weights = nullptr, bool set = false) {
     if (!ws) return VG_ERR_INVALID_ARG;
     if (ws->stage < 3) return fail(ws, VG_ERR_STATE, "vg_render_bwd before vg_render_fwd");
     if ((!dL_drgb && ws->n_pixels > 0 && !drgb_optional) || (ws->g.n > 0 && (!dmu || !dscale || !dquat || !dkappa)))
@@ -762,7 +762,7 @@ static vg_status render_bwd_impl(vg_workspace *ws, const float *dL_drgb, const f
     {
         // the chain writes every Gaussian's gradient: overwriting with VG_FLAG_GRAD_ZERO, else adding
         ProfScope ps(ws, ST_CHAIN, st);
-        VG_CUDA(ws, launch_chain(ws->g, ws->views.p, ws->n_views, ws->grad.p, (ws->opts.flags & VG_FLAG_GRAD_ZERO) ? 1 : 0,
+        VG_CUDA(ws, launch_chain(ws->g, ws->views.p, ws->n_views, ws->grad.p, set || (ws->opts.flags & VG_FLAG_GRAD_ZERO) ? 1 : 0,
                                  dmu, dscale, dquat, dkappa, dsh, st, &ws->launches));
     }
     ws->grad_zero_p = ws->grad.p;   // the chain left the accumulator zero
@@ -773,6 +773,11 @@ static vg_status render_bwd_impl(vg_workspace *ws, const float *dL_drgb, const f
 vg_status vg_render_bwd(vg_workspace *ws, const float *dL_drgb, const float *dL_dT, float *dmu, float *dscale,
                         float *dquat, float *dkappa, float *dsh, void *stream) {
     return render_bwd_impl(ws, dL_drgb, dL_dT, dmu, dscale, dquat, dkappa, dsh, stream, false);
+}
+
+vg_status vg_render_bwd_set(vg_workspace *ws, const float *dL_drgb, const float *dL_dT, float *dmu, float *dscale,
+                            float *dquat, float *dkappa, float *dsh, void *stream) {
+    return render_bwd_impl(ws, dL_drgb, dL_dT, dmu, dscale, dquat, dkappa, dsh, stream, false, nullptr, true);
 }
 
 vg_status vg_project_cone(vg_workspace *ws, const vg_gaussians *g, const vg_camera *cams, int32_t n_views,
@@ -1055,6 +1060,7 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
     const bool fused = target != nullptr;
     const bool backward = dL_dproj != nullptr || fused;
     const bool proj_given = dL_dproj && !fused && (opts && (opts->flags & VG_FLAG_PROJ_GIVEN));
+    const bool lists = !proj_given || !(opts->flags & VG_FLAG_NO_LISTS);   // the projection alone needs them
     VG_TRY(check_gauss(ws, g, false));
     if (!beam || beam->n_angles < 1 || !beam->angles || beam->det_w <= 0 || beam->det_h <= 0 ||
         !finite_pos(beam->pitch_u) || !finite_pos(beam->pitch_v) || !std::isfinite(beam->u0) ||
@@ -1114,8 +1120,10 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
             vh[v].tile_base = (int)(v * tpv);
             vh[v].pix_base = (long long)v * det_px;
         }
-        VG_TRY(ensure(ws, ws->views, vh.size(), "views"));
-        VG_CUDA(ws, cudaMemcpyAsync(ws->views.p, vh.data(), vh.size() * sizeof(ViewInfo), cudaMemcpyHostToDevice, st));
+        if (lists) {
+            VG_TRY(ensure(ws, ws->views, vh.size(), "views"));
+            VG_CUDA(ws, cudaMemcpyAsync(ws->views.p, vh.data(), vh.size() * sizeof(ViewInfo), cudaMemcpyHostToDevice, st));
+        }
         // the backward's item order: by the tile of the footprint's centre (the last key: no footprint), once a
         // view's weights no longer fit one SM's L1
         const bool by_home = backward && (long long)beam->det_h * tomo_pitch(beam->det_w) * 4 > kTomoL1Image;
@@ -1128,31 +1136,33 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
                                                ws->rec.p, ws->count.p, ws->rect.p, by_home ? home : nullptr, st,
                                                &ws->launches));
         }
-        {
-            ProfScope ps(ws, ST_SCAN, st);
-            VG_CUDA(ws, launch_scan_gather(ws->count.p, nullptr, ws->offsets.p, items, ws->scan_tmp.p,
-                                           total64_ptr(ws), ~0ull, lookback_err_ptr(ws), false, st, &ws->launches));
-        }
-        long long total = 0;
-        VG_TRY(read_total(ws, st, &total));
-        if (total > (long long)(1u << 30) - 1)
-            return fail(ws, VG_ERR_INVALID_ARG, "more than 2^30 - 1 (tile, Gaussian) instances in an angle batch");
-        VG_TRY(reserve_instances(ws, total));
-        {
-            ProfScope ps(ws, ST_DUP, st);
-            VG_CUDA(ws, launch_duplicate(nullptr, ws->offsets.p, ws->rect.p, ws->views.p, items, N > 0 ? N : 1,
-                                         ws->ikey[0].p, ws->ival[0].p, ws->capacity, st, &ws->launches));
-        }
-        {
-            ProfScope ps(ws, ST_TILE, st);
-            VG_CUDA(ws, launch_radix_sort(ws->ikey[0].p, ws->ival[0].p, ws->ikey[1].p, ws->ival[1].p, ws->ikey[0].p,
-                                          ws->ival[0].p, total, nullptr, bits_for(n_tiles), ws->hist.p,
-                                          lookback_err_ptr(ws), false, &ws->inst_key, &ws->inst_item, st, &ws->launches));
-        }
-        VG_TRY(ensure(ws, ws->ranges, (size_t)n_tiles, "tile ranges"));
-        {
-            ProfScope ps(ws, ST_RANGES, st);
-            VG_CUDA(ws, launch_ranges(ws->inst_key, total, nullptr, ws->ranges.p, n_tiles, false, st, &ws->launches));
+        long long total = ws->n_inst;
+        if (lists) {
+            {
+                ProfScope ps(ws, ST_SCAN, st);
+                VG_CUDA(ws, launch_scan_gather(ws->count.p, nullptr, ws->offsets.p, items, ws->scan_tmp.p,
+                                               total64_ptr(ws), ~0ull, lookback_err_ptr(ws), false, st, &ws->launches));
+            }
+            VG_TRY(read_total(ws, st, &total));
+            if (total > (long long)(1u << 30) - 1)
+                return fail(ws, VG_ERR_INVALID_ARG, "more than 2^30 - 1 (tile, Gaussian) instances in an angle batch");
+            VG_TRY(reserve_instances(ws, total));
+            {
+                ProfScope ps(ws, ST_DUP, st);
+                VG_CUDA(ws, launch_duplicate(nullptr, ws->offsets.p, ws->rect.p, ws->views.p, items, N > 0 ? N : 1,
+                                             ws->ikey[0].p, ws->ival[0].p, ws->capacity, st, &ws->launches));
+            }
+            {
+                ProfScope ps(ws, ST_TILE, st);
+                VG_CUDA(ws, launch_radix_sort(ws->ikey[0].p, ws->ival[0].p, ws->ikey[1].p, ws->ival[1].p, ws->ikey[0].p,
+                                              ws->ival[0].p, total, nullptr, bits_for(n_tiles), ws->hist.p,
+                                              lookback_err_ptr(ws), false, &ws->inst_key, &ws->inst_item, st, &ws->launches));
+            }
+            VG_TRY(ensure(ws, ws->ranges, (size_t)n_tiles, "tile ranges"));
+            {
+                ProfScope ps(ws, ST_RANGES, st);
+                VG_CUDA(ws, launch_ranges(ws->inst_key, total, nullptr, ws->ranges.p, n_tiles, false, st, &ws->launches));
+            }
         }
         float *proj_b = proj + (size_t)a0 * det_px;
         if (!proj_given) {
@@ -1188,7 +1198,7 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
         ws->n_pixels = (long long)nb * det_px;
     }
     ws->stage = 0;
-    ws->tomo_read = true;
+    if (lists) ws->tomo_read = true;
     return VG_OK;
 }
 
