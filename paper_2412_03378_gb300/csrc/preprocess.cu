@@ -1,7 +1,7 @@
 // Per-(view, Gaussian) preprocessing: key function (depth key + conservative tile
 // rectangle), view-dependent colour and the blend record.  One thread per item, a warp per 32
 // consecutive Gaussians of one view.  The SH rows come in through shared memory so that the HBM
-// reads (the kernel's bound) are coalesced: FP32 degree-3 rows (SH3) as 16-byte pieces, other rows
+// reads (the kernel's bound) are coalesced: degree-3 rows (SH3) as 16-byte pieces, other rows
 // element by element.  Each visible item's 96-byte record goes out from registers as six 16-byte
 // stores (records of culled items are never read and are not written).
 #include "geometry.cuh"
@@ -34,7 +34,7 @@ k_preprocess(GaussIn g, const ViewInfo *__restrict__ views, int n_views, float z
         // the SH rows of the warp's Gaussians, coalesced, before (and independent of) the key; the
         // parameter loads are issued before the wait so that both round trips overlap
         if (SH3)
-            warp_load_sh3((const float *)g.sh + gbase * K3, nloc, reinterpret_cast<float4 *>(buf), lane);
+            warp_load_sh3((const ST *)g.sh + gbase * K3, nloc, reinterpret_cast<float4 *>(buf), lane);
         else if (g.sh)
             warp_load_rows<ST>((const ST *)g.sh + gbase * K3, nloc, K3, buf, lane);
         float mu[3], s[3], q[4], kin;
@@ -122,8 +122,8 @@ static cudaError_t launch_pre_t(const GaussIn &g, const ViewInfo *views_d, int n
     long long blocks = (chunks + kPreWarps - 1) / kPreWarps;
     if (blocks > 152 * 64) blocks = 152 * 64;
     if (blocks < 1) blocks = 1;
-    // FP32 degree-3 SH rows of a 16-byte aligned array: 16-byte copies
-    if (sh3_rows<ST>(g))
+    // degree-3 SH rows of a 16-byte aligned array: 16-byte copies
+    if (sh3_rows(g))
         pdl_launch(k_preprocess<RT, ST, true>, (unsigned)blocks, 32 * kPreWarps, 0, st, g, views_d, n_views, z_near,
                    tau_cut, rec, depth, count, rect, prect, n_visible);
     else

@@ -505,7 +505,7 @@ k_chain(GaussIn g, const ViewInfo *__restrict__ views, int n_views, float *__res
         float *__restrict__ dsh) {
     pdl_entry();
     // SH coefficients (as float) and the SH gradient being accumulated: kRowStride floats per row,
-    // or (SH3: FP32 degree-3 rows and a 16-byte aligned dsh) kRow16 float4 per row
+    // or (SH3: degree-3 rows and a 16-byte aligned dsh) kRow16 float4 per row
     constexpr int kStride = SH3 ? 4 * kRow16 : kRowStride;
     __shared__ __align__(16) float ssh[kChainWarps][32 * kStride];
     __shared__ __align__(16) float sdsh[kChainWarps][32 * kStride];
@@ -518,7 +518,7 @@ k_chain(GaussIn g, const ViewInfo *__restrict__ views, int n_views, float *__res
         const int nloc = (int)min(32LL, (long long)g.n - gbase);
         const long long gi = gbase + lane;
         if (SH3) {
-            warp_load_sh3((const float *)g.sh + gbase * K3, nloc, reinterpret_cast<float4 *>(ssh[wi]), lane);
+            warp_load_sh3((const ST *)g.sh + gbase * K3, nloc, reinterpret_cast<float4 *>(ssh[wi]), lane);
             if (zero) {
 #pragma unroll
                 for (int j = 0; j < kSh3Pieces; ++j)
@@ -774,8 +774,8 @@ static cudaError_t launch_chain_t(const GaussIn &g, const ViewInfo *views_d, int
     long long b = ((long long)g.n + 32 * kChainWarps - 1) / (32 * kChainWarps);
     if (b > 152 * 64) b = 152 * 64;
     if (b < 1) b = 1;
-    // FP32 degree-3 SH rows and a 16-byte aligned SH gradient: 16-byte pieces
-    const bool sh3 = sh3_rows<ST>(g) && dsh != nullptr && ((uintptr_t)dsh & 15u) == 0;
+    // degree-3 SH rows and a 16-byte aligned SH gradient: 16-byte pieces
+    const bool sh3 = sh3_rows(g) && dsh != nullptr && ((uintptr_t)dsh & 15u) == 0;
 #define VG_CHAIN_LAUNCH(SPL, S3)                                                                                     \
     pdl_launch(k_chain<RT, ST, SPL, S3>, (unsigned)b, 32 * kChainWarps, 0, st, g, views_d, n_views, grad_acc, zero, dmu, \
                dscale, dquat, dkappa, dsh)
