@@ -3,6 +3,8 @@
 // the two kernels compute identical bits and therefore take identical skip decisions.
 #pragma once
 
+#include <type_traits>
+
 #include "vg_internal.cuh"
 
 namespace vg {
@@ -155,6 +157,16 @@ __device__ __forceinline__ bool box_inside(const WarpBox &b, const short4 &r) {
 
 __device__ __forceinline__ bool pixel_outside(int x, int y, const short4 &r) {
     return (x < r.x) | (x > r.z) | (y < r.y) | (y > r.w);   // no branches: the caller's evaluation stays in line
+}
+
+// The forward's staged footprints: short4 as in memory, or int4 (x0, y0, width - 1, height - 1).
+__device__ __forceinline__ void put_rect(short4 &d, const short4 &r) { d = r; }
+__device__ __forceinline__ void put_rect(int4 &d, const short4 &r) { d = make_int4(r.x, r.y, r.z - r.x, r.w - r.y); }
+__device__ __forceinline__ bool box_misses(const WarpBox &b, const int4 &r) {
+    return r.x + r.z < b.x0 || r.x > b.x1 || r.y + r.w < b.y0 || r.y > b.y1;
+}
+__device__ __forceinline__ bool pixel_in(int x, int y, const int4 &r) {
+    return ((unsigned)(x - r.x) <= (unsigned)r.z) & ((unsigned)(y - r.y) <= (unsigned)r.w);
 }
 
 // Conservative opacity test of one record against a warp's pixel box, for blending with

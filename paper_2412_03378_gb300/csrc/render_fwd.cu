@@ -40,7 +40,10 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
     constexpr int kChunk = CH;   // records per barrier
     constexpr int kRF4 = RecOf<SPLAT>::kF4, kCF4 = kCullF4<SPLAT>;
     __shared__ float4 srec[kChunk * kRF4];
-    __shared__ short4 srect[kChunk];
+    // footprints; where every pixel is tested, as (first x, first y, width - 1, height - 1) in 32 bits: a subtraction and an
+    // unsigned comparison per axis, nothing to unpack
+    using Rect = std::conditional_t<PIXTEST, int4, short4>;
+    __shared__ Rect srect[kChunk];
     __shared__ float4 scull[PIXTEST ? 1 : kChunk * kCF4];   // Gram matrices for the opacity test
     // per record, contiguous for the opacity test: (px0, py0, log2 K, |A0|) and |A1|
     __shared__ float4 sref[PIXTEST ? 1 : kChunk];
@@ -86,7 +89,7 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                 q[k] = __ldg(src + k);
                 srec[r * kRF4 + k] = q[k];
             }
-            srect[r] = prect[item];
+            put_rect(srect[r], prect[item]);
             if (!PIXTEST) {
                 float4 c[kCF4];
                 cull_row<SPLAT>(q, c, sref[r], ssq1[r]);
@@ -121,10 +124,7 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                     for (int i = 0; i < kIlp; ++i) {
                         typename RecOf<SPLAT>::type r;
                         load_rec(&srec[js[i] * kRF4], r);
-                        if (PIXTEST) {
-                            const short4 pr = srect[js[i]];
-                            in[i] = in[i] & !pixel_outside(x0, y0, pr);
-                        }
+                        if constexpr (PIXTEST) in[i] = in[i] & pixel_in(x0, y0, srect[js[i]]);
                         if constexpr (SPLAT) {   // Eq. 6: alpha = min(o G'(p), alpha_max)
                             SplatCol sc;
                             splat_col(r, xf, sc);
@@ -175,15 +175,14 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                 if constexpr (P > 1 && SPLAT) {
                     SplatRec r;
                     load_rec(&srec[j * kRF4], r);
-                    short4 pr;
-                    if (PIXTEST) pr = srect[j];
+                    const Rect pr = srect[j];
                     SplatCol sc[P / 2];   // pixel columns of the thread
 #pragma unroll
                     for (int c = 0; c < P / 2; ++c) splat_col(r, c ? xf + 1.0f : xf, sc[c]);
 #pragma unroll
                     for (int k = 0; k < P; ++k) {   // Eq. 6: alpha = min(o G'(p), alpha_max)
                         bool valid = (live >> k) & 1u;
-                        if (PIXTEST) valid = valid && !pixel_outside(x0 + L::ox(k), y0 + L::oy(k), pr);
+                        if constexpr (PIXTEST) valid = valid & pixel_in(x0 + L::ox(k), y0 + L::oy(k), pr);
                         float dx, dy, q;
                         const float a_c =
                             fminf(splat_at(r, sc[L::ox(k)], L::oy(k) ? yf + (float)L::oy(k) : yf, dx, dy, q), bp.alpha_max);
@@ -220,8 +219,7 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                     for (int i = 0; i < kN; ++i) {
                         RecPairs r;
                         load_rec(&srec[js[i] * kRF4], r);
-                        short4 pr;
-                        if (PIXTEST) pr = srect[js[i]];
+                        const Rect pr = srect[js[i]];
 #pragma unroll
                         for (int c = 0; c < P / 2; ++c) {
                             ColBase cb;
@@ -230,11 +228,12 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                             pair_tau2(r, cb, f2_pack(yf, yf + 1.0f), f2_pack(Lp[c], Lp[c + kRow]), t[i][c]);
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
-                                bool ok = kN == 1 ? ((live >> (c + h * kRow)) & 1u) != 0 : in[i];
-                                if (PIXTEST) ok = ok & !pixel_outside(x0 + c, y0 + h, pr);
+                                // (no pixel of the projection finishes, and footprints end at the image's edge)
+                                bool ok = CONE ? true : (kN == 1 ? ((live >> (c + h * kRow)) & 1u) != 0 : in[i]);
+                                if constexpr (PIXTEST) ok = ok & pixel_in(x0 + c, y0 + h, pr);
                                 if (COUNT) pairs += ok & ((live >> (c + h * kRow)) & 1u);
                                 const float t_c = fminf(t[i][c][h], bp.tau_max);
-                                v[i][c][h] = ok & (t_c >= bp.tau_skip);
+                                v[i][c][h] = CONE ? ok : ok & (t_c >= bp.tau_skip);   // tau_skip = 0, and t_c is no NaN
                                 t[i][c][h] = v[i][c][h] ? t_c : 0.0f;
                             }
                             if (!CONE) {
