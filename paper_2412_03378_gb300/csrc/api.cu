@@ -588,7 +588,12 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
     VG_TRY(ensure(ws, ws->tord, (size_t)ws->n_tiles, "tile order"));
     // the tile sort's scratch: its own where the capacity is known and it may be had, so that it is cleared in advance
     const size_t tile_words = known ? radix_scratch_words(ws->capacity, 32) : 0;
-    const bool own = known && (ws->hist_tile.n >= tile_words || !fixed || !ws->hist_tile.p);
+    bool own = known && (ws->hist_tile.n >= tile_words || !fixed || !ws->hist_tile.p);
+    if (own && ws->hist_tile.n < tile_words) {   // a capturing stream allocates nothing here
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        VG_CUDA(ws, cudaStreamIsCapturing(st, &cap));
+        own = cap == cudaStreamCaptureStatusNone;
+    }
     if (own) VG_TRY(ensure(ws, ws->hist_tile, tile_words, "radix sort scratch"));
     // 1. items by depth key (stable: ties keep index order)
     {
@@ -673,6 +678,7 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
             // the binning enqueued ahead still uses the buffers about to be replaced
             if (ahead) VG_CUDA(ws, cudaStreamSynchronize(st));
             VG_TRY(reserve_instances(ws, total));
+            VG_TRY(ensure(ws, ws->hist_tile, radix_scratch_words(ws->capacity, 32), "radix sort scratch"));   // for the next call
             VG_TRY(bin_rest(total, nullptr, false));
         }
         ws->n_inst = total;
