@@ -45,3 +45,31 @@ def test_one_workspace_over_sizes(gpu_lib):
         _check(vg, ws, _scene(n, 400 + n), cams)
     for n, cams in ((9000, two), (40, one), (20000, one)):
         _check(vg, ws, _scene(n, 400 + n), cams, flags=vg.FLAG_FIXED_CAPACITY)
+
+
+@pytest.mark.parametrize("n", [300, 20000])
+def test_fixed_capacity_captured_after_a_plain_binning(gpu_lib, n):
+    """A step with a fixed capacity captured right after one plain step (nothing reserved): the scratch is there."""
+    import torch
+
+    vg = gpu_lib
+    sc, cam = _scene(n, 500 + n), [synth.look_at((0.0, 0.0, -4.0), (0, 0, 0), 64, 48, 50.0)]
+    g, ws = dev_scene(vg, sc), vg.Workspace()
+    out = torch.empty((64 * 48, 3), device="cuda:0")
+
+    def step(flags):
+        ws.preprocess(g, cam, vg_opts(vg, dict(oracle.COMPAT), flags))
+        ws.bin_sort()
+        ws.render_fwd(out)
+
+    step(0)
+    want = out.clone()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step(vg.FLAG_FIXED_CAPACITY)
+    for _ in range(2):
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
