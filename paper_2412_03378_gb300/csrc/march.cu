@@ -22,7 +22,7 @@
 // longest list in sequence were the whole 2.80 ms.  With no early stop (T_stop = 0) the passes of a
 // pixel are independent up to their transmittance, so they are spread over groups of CTAs, each
 // leaving its colour and transmittance per pixel, which k_march_combine strings together.  A frame
-// of that size and its march: 2.78 -> 0.48 ms (the march 2.80 -> 0.34 ms).
+// of that size and its march: 2.83 -> 0.39 ms (the march 2.80 -> 0.31 ms).
 #include "blend.cuh"
 #include "geometry.cuh"
 
@@ -156,7 +156,8 @@ k_ray_march(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vie
                     float a, qq;
                     f2_unpack(pair_squares(R, col, dy), a, qq);
                     const float bq = fmaf(e4.x, dx, fmaf(e4.y, dy, e4.z));
-                    const float ia = 1.0f / a;
+                    float ia = rcp_approx(a);   // and one Newton step, in place of the rounded division's dozen instructions
+                    ia = fmaf(ia, fmaf(-a, ia, 1.0f), ia);
                     const float lp = fmaf(-qq * ia, kHalfLog2e, r5.x - kLog2Sqrt2Pi);   // log2(kappa exp(-m^2/2))
                     const float gam = -bq * dcn * ia;
                     const float h = hscale * a;                                          // log2(e) / (2 beta^2)
