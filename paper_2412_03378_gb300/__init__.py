@@ -238,8 +238,8 @@ class Gaussians:
 def camera_struct(cam):
     """Any object with R (3x3), t (3), fx, fy, cx, cy, width, height."""
     c = _Camera()
-    c.R[:] = [float(x) for row in cam.R for x in row]
-    c.t[:] = [float(x) for x in cam.t]
+    c.R[:] = [float(x) for row in cam.R for x in row][:9]
+    c.t[:] = [float(cam.t[k]) for k in range(3)]   # t may be homogeneous
     c.fx, c.fy, c.cx, c.cy = float(cam.fx), float(cam.fy), float(cam.cx), float(cam.cy)
     c.width, c.height = int(cam.width), int(cam.height)
     return c
