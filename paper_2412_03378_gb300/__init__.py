@@ -492,12 +492,14 @@ class _TomoFn(torch.autograd.Function):
     alone while they are the forward's; parameters written to in between are projected anew."""
 
     @staticmethod
-    def forward(ctx, ws, beam, opts, mu, scale, quat, kappa):
+    def forward(ctx, ws, beam, opts, keep, mu, scale, quat, kappa):
         g = Gaussians(mu.detach().contiguous(), scale.detach().contiguous(), quat.detach().contiguous(),
                       kappa.detach().contiguous(), None, 0)
         proj = torch.empty((len(beam.angles), int(beam.det_h), int(beam.det_w)), device=mu.device,
                            dtype=torch.float32)
         ws.project_tomo(g, beam, opts, proj)
+        if not keep:   # no backward can come (and a tensor of inference mode has no version counter)
+            return proj
         ctx.ws, ctx.beam, ctx.opts, ctx.g, ctx.gen = ws, beam, opts, g, ws.generation
         ctx.seen = [t._version for t in (g.mu, g.scale, g.quat, g.kappa)]
         ctx.angles = [float(a) for a in beam.angles]
@@ -527,7 +529,7 @@ class _TomoFn(torch.autograd.Function):
         o = copy.copy(opts)
         o.flags = flags
         ctx.ws.project_tomo(g, beam, o, proj, g_proj.contiguous().float(), *grads)
-        return (None, None, None) + tuple(d.to(t.dtype) for d, t in zip(grads, params))
+        return (None, None, None, None) + tuple(d.to(t.dtype) for d, t in zip(grads, params))
 
 
 class _ConeFn(torch.autograd.Function):
@@ -561,7 +563,8 @@ class Projector:
 
     def parallel(self, mu, scale, quat, kappa, beam):
         """proj [A, det_h, det_w] = exp(-sum of the line integrals)."""
-        return _TomoFn.apply(self.ws, beam, self.opts, mu, scale, quat, kappa)
+        keep = torch.is_grad_enabled() and any(t.requires_grad for t in (mu, scale, quat, kappa))
+        return _TomoFn.apply(self.ws, beam, self.opts, keep, mu, scale, quat, kappa)
 
     def cone(self, mu, scale, quat, kappa, cams: Sequence):
         """proj [sum H*W] over the cameras' detectors."""

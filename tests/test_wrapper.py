@@ -16,3 +16,67 @@ def test_camera_translation_may_be_homogeneous(t):
     assert list(c.t) == [1.0, 2.0, 3.0] and list(c.R) == [1, 0, 0, 0, 1, 0, 0, 0, 1]
     cam.R = [[1, 0, 0], [0, 1, 0], [0, 0, 1], [7, 7, 7]]
     assert list(vg.camera_struct(cam).R) == [1, 0, 0, 0, 1, 0, 0, 0, 1]
+
+
+class StandIn:
+    """A workspace that records its calls and writes ones into the outputs, of which the library writes `rows` rows."""
+
+    def __init__(self, rows=None):
+        self.generation, self.calls, self.rows = 0, [], rows
+
+    def _fill(self, tensors):
+        for t in tensors:
+            if t is not None:
+                t.view(-1)[:t.numel() if self.rows is None else self.rows * max(1, t[0].numel())] = 1.0
+
+    def project_tomo(self, g, beam, opts, proj, dL=None, *grads, stream=None):
+        self.generation += 1
+        self.calls.append((opts.flags, dL))
+        proj.fill_(0.5)
+        self._fill(grads)
+
+    def preprocess(self, g, cams, opts, stream=None):
+        self.generation += 1
+
+    def bin_sort(self, stream=None):
+        pass
+
+    def render_fwd(self, rgb, T=None, stream=None):
+        rgb.fill_(0.25)
+        T.fill_(0.5)
+
+    def render_bwd_set(self, dL_drgb, dL_dT, *grads, stream=None):
+        self.calls.append((dL_drgb, dL_dT))
+        self._fill(grads)
+
+    def query(self):
+        raise AssertionError("a query synchronises")
+
+
+def _params(n=5, sh=4):
+    import torch
+    return [torch.rand(s) for s in ((n, 3), (n, 3), (n, 4), (n,), (n, sh, 3))]
+
+
+def _beam():
+    return SimpleNamespace(angles=[0.0, 1.0], det_w=6, det_h=4, pitch_u=0.1, pitch_v=0.1, u0=0.0, v0=0.0)
+
+
+@pytest.fixture
+def stand_in(monkeypatch):
+    ws = StandIn()
+    monkeypatch.setattr(vg, "Workspace", lambda: ws)
+    return ws
+
+
+@pytest.mark.parametrize("how", ["inference", "inference leaf", "no_grad"])
+def test_parallel_without_a_gradient(stand_in, how):
+    """Computed parameters under inference mode have no version counter; nothing is kept for a backward that cannot come."""
+    import torch
+    pro, (mu, ls, q, k, _) = vg.Projector(), _params()
+    mu.requires_grad_(how == "no_grad")
+    with torch.no_grad() if how == "no_grad" else torch.inference_mode():
+        if how == "inference leaf":
+            mu = torch.rand((5, 3))
+        proj = pro.parallel(mu, ls.exp(), torch.nn.functional.normalize(q, dim=1), k, _beam())
+    assert proj.shape == (2, 4, 6) and float(proj.min()) == 0.5
