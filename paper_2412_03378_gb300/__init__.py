@@ -457,6 +457,14 @@ def n_pixels(cams):
     return sum(int(c.width) * int(c.height) for c in cams)
 
 
+def _grad_buffers(g: Gaussians, *params):
+    """Buffers for gradients that the library overwrites; cleared where a parameter holds more than the library reads
+    (rows beyond g.n, coefficients beyond sh_degree's), whose gradient is zero."""
+    per_row = (3, 3, 4, 1, 3 * (g.sh_degree + 1) ** 2)
+    return [(torch.empty_like if t.numel() == g.n * k else torch.zeros_like)(t, dtype=torch.float32)
+            for t, k in zip(params, per_row)]
+
+
 class _RenderFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, ws, cams, opts, sh_degree, mu, scale, quat, kappa, sh):
@@ -477,8 +485,7 @@ class _RenderFn(torch.autograd.Function):
         ws, g = ctx.ws, ctx.g
         if ws.generation != ctx.gen:
             raise RuntimeError("the workspace was reused by another forward before this backward")
-        dmu, dscale, dquat, dkappa, dsh = (torch.empty_like(t, dtype=torch.float32)
-                                           for t in (g.mu, g.scale, g.quat, g.kappa, g.sh))
+        dmu, dscale, dquat, dkappa, dsh = _grad_buffers(g, g.mu, g.scale, g.quat, g.kappa, g.sh)
         g_rgb = (g_rgb if g_rgb is not None else torch.zeros((n_pixels_ws(ws), 3), device=g.mu.device)).contiguous()
         g_T = g_T.contiguous() if g_T is not None else None
         ws.render_bwd_set(g_rgb.float(), None if g_T is None else g_T.float(), dmu, dscale, dquat, dkappa, dsh)
@@ -515,7 +522,7 @@ class _TomoFn(torch.autograd.Function):
     def backward(ctx, g_proj):
         g, beam, opts = ctx.g, ctx.beam, ctx.opts
         params = (g.mu, g.scale, g.quat, g.kappa)
-        grads = [torch.empty_like(t, dtype=torch.float32) for t in params]
+        grads = _grad_buffers(g, *params)
         flags = opts.flags | FLAG_GRAD_ZERO
         same = ctx.proj is not None and ctx.seen == [t._version for t in params] and \
             ctx.geometry == (int(beam.det_w), int(beam.det_h), float(beam.pitch_u), float(beam.pitch_v), float(beam.u0),

@@ -80,3 +80,23 @@ def test_parallel_without_a_gradient(stand_in, how):
             mu = torch.rand((5, 3))
         proj = pro.parallel(mu, ls.exp(), torch.nn.functional.normalize(q, dim=1), k, _beam())
     assert proj.shape == (2, 4, 6) and float(proj.min()) == 0.5
+
+
+def test_gradients_of_what_the_library_does_not_write(monkeypatch):
+    """Rows beyond the Gaussians that mu counts, and coefficients beyond sh_degree's, have gradient zero."""
+    import torch
+    n = 3
+    ws = StandIn(rows=n)
+    monkeypatch.setattr(vg, "Workspace", lambda: ws)
+    empty = torch.empty_like
+    monkeypatch.setattr(torch, "empty_like", lambda *a, **k: empty(*a, **k).fill_(float("nan")))
+    mu, scale, quat, kappa, _ = _params(n + 2)
+    mu = mu[:n].contiguous().requires_grad_(True)
+    scale, quat, kappa = (t.requires_grad_(True) for t in (scale, quat, kappa))
+    for got in torch.autograd.grad(vg.Projector().parallel(mu, scale, quat, kappa, _beam()).sum(), (mu, scale, quat, kappa)):
+        assert torch.equal(got[:n], torch.ones_like(got[:n])) and float(got[n:].abs().sum()) == 0.0
+    sh = torch.rand((n, 16, 3), requires_grad=True)
+    cams = [SimpleNamespace(width=4, height=3)]
+    ws._fill = lambda ts: [t.view(-1)[:t.numel() if t.dim() < 3 else 4 * n * 3].fill_(1.0) for t in ts]
+    rgb, _ = vg.Rasterizer().render(mu, scale, quat, kappa, sh, cams, sh_degree=1)
+    assert float(torch.autograd.grad(rgb.sum(), sh)[0].sum()) == 4 * n * 3
