@@ -477,7 +477,8 @@ class _RenderFn(torch.autograd.Function):
         ws.bin_sort()
         ws.render_fwd(rgb, T)
         ctx.ws, ctx.gen, ctx.g = ws, ws.generation, g
-        ctx.set_materialize_grads(False)   # an output the loss does not use costs nothing
+        ctx.pixels = P
+        ctx.set_materialize_grads(False)   # no zeros are made for a T that the loss does not use
         return rgb, T
 
     @staticmethod
@@ -486,7 +487,7 @@ class _RenderFn(torch.autograd.Function):
         if ws.generation != ctx.gen:
             raise RuntimeError("the workspace was reused by another forward before this backward")
         dmu, dscale, dquat, dkappa, dsh = _grad_buffers(g, g.mu, g.scale, g.quat, g.kappa, g.sh)
-        g_rgb = (g_rgb if g_rgb is not None else torch.zeros((n_pixels_ws(ws), 3), device=g.mu.device)).contiguous()
+        g_rgb = (g_rgb if g_rgb is not None else torch.zeros((ctx.pixels, 3), device=g.mu.device)).contiguous()
         g_T = g_T.contiguous() if g_T is not None else None
         ws.render_bwd_set(g_rgb.float(), None if g_T is None else g_T.float(), dmu, dscale, dquat, dkappa, dsh)
         return (None, None, None, None, dmu.to(g.mu.dtype), dscale.to(g.scale.dtype), dquat.to(g.quat.dtype),

@@ -100,3 +100,13 @@ def test_gradients_of_what_the_library_does_not_write(monkeypatch):
     ws._fill = lambda ts: [t.view(-1)[:t.numel() if t.dim() < 3 else 4 * n * 3].fill_(1.0) for t in ts]
     rgb, _ = vg.Rasterizer().render(mu, scale, quat, kappa, sh, cams, sh_degree=1)
     assert float(torch.autograd.grad(rgb.sum(), sh)[0].sum()) == 4 * n * 3
+
+
+def test_render_backward_of_T_alone(stand_in):
+    """A loss of T alone asks the device nothing (the stand-in's query raises) and hands over a zero dL/drgb."""
+    import torch
+    params = [p.requires_grad_(True) for p in _params()]
+    _, T = vg.Rasterizer().render(*params, [SimpleNamespace(width=4, height=3), SimpleNamespace(width=2, height=1)])
+    torch.autograd.grad(T.sum(), params)
+    drgb, dT = stand_in.calls[-1]
+    assert drgb.shape == (14, 3) and not drgb.any() and torch.equal(dT, torch.ones(14))
