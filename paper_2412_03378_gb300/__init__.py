@@ -343,10 +343,10 @@ class Workspace:
         b.det_w, b.det_h = int(beam.det_w), int(beam.det_h)
         b.pitch_u, b.pitch_v, b.u0, b.v0 = float(beam.pitch_u), float(beam.pitch_v), float(beam.u0), float(beam.v0)
         oc = opts.c()
-        self.generation += 1
         self._chk(self._L.vg_project_tomo(self.h, ctypes.byref(g.c()), ctypes.byref(b), ctypes.byref(oc), _ptr(proj),
                                           _ptr(dL_dproj), _ptr(dmu), _ptr(dscale), _ptr(dquat), _ptr(dkappa),
                                           _stream(stream)))
+        self.generation += 1
 
     def tomo_l2_step(self, g: Gaussians, beam, opts: Opts, target, scale, proj, loss, dmu, dscale, dquat, dkappa,
                      stream=None):
@@ -357,10 +357,10 @@ class Workspace:
         b.det_w, b.det_h = int(beam.det_w), int(beam.det_h)
         b.pitch_u, b.pitch_v, b.u0, b.v0 = float(beam.pitch_u), float(beam.pitch_v), float(beam.u0), float(beam.v0)
         oc = opts.c()
-        self.generation += 1
         self._chk(self._L.vg_tomo_l2_step(self.h, ctypes.byref(g.c()), ctypes.byref(b), ctypes.byref(oc), _ptr(target),
                                           float(scale), _ptr(proj), _ptr(loss), _ptr(dmu), _ptr(dscale), _ptr(dquat),
                                           _ptr(dkappa), _stream(stream)))
+        self.generation += 1
 
     def project_cone(self, g: Gaussians, cams, opts: Opts, proj, dL_dproj=None, dmu=None, dscale=None, dquat=None,
                      dkappa=None, stream=None):
@@ -379,9 +379,9 @@ class Workspace:
             gr.origin[a], gr.voxel[a] = float(origin[a]), float(voxel[a])
         gr.nx, gr.ny, gr.nz = (int(d) for d in dims)
         oc = opts.c()
-        self.generation += 1
         self._chk(self._L.vg_query_density(self.h, ctypes.byref(g.c()), ctypes.byref(gr), ctypes.byref(oc), _ptr(out),
                                            _stream(stream)))
+        self.generation += 1
 
     def ray_march(self, t_near, t_far, n_samples, rgb=None, T=None, raster_rgb=None, err_map=None, stream=None):
         """Ray-marching reference of the binned views (see vg_ray_march): rgb [P, 3], T [P] and the

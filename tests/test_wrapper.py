@@ -110,3 +110,25 @@ def test_render_backward_of_T_alone(stand_in):
     torch.autograd.grad(T.sum(), params)
     drgb, dT = stand_in.calls[-1]
     assert drgb.shape == (14, 3) and not drgb.any() and torch.equal(dT, torch.ones(14))
+
+
+@pytest.mark.parametrize("call", ["project_tomo", "tomo_l2_step", "query_density"])
+def test_refused_call_leaves_the_outstanding_forward(call):
+    """A call that the library refuses for its arguments has not touched the workspace."""
+    import ctypes
+
+    ws = vg.Workspace.__new__(vg.Workspace)
+    ws.h, ws.generation = None, 7
+    refuse = lambda *a: 1
+    ws._L = SimpleNamespace(vg_project_tomo=refuse, vg_tomo_l2_step=refuse, vg_query_density=refuse,
+                            vg_last_error=lambda h: b"refused")
+    g = SimpleNamespace(c=lambda: ctypes.c_int(0))
+    args = {"project_tomo": (g, _beam(), vg.Opts(), None), "query_density": (g, (0, 0, 0), (1, 1, 1), (1, 1, 1), vg.Opts(), None),
+            "tomo_l2_step": (g, _beam(), vg.Opts(), None, 1.0, None, None, None, None, None, None)}[call]
+    stream, vg._stream = vg._stream, lambda s=None: None
+    try:
+        with pytest.raises(vg.VGError):
+            getattr(ws, call)(*args)
+    finally:
+        vg._stream = stream
+    assert ws.generation == 7
