@@ -151,8 +151,9 @@ typedef struct {
                                       projection of the same Gaussians, beam and options (from an
                                       earlier call), so it is not recomputed before the backward */
 #define VG_FLAG_NO_LISTS 64u       /* with VG_FLAG_PROJ_GIVEN: the tile lists, which the gradient
-                                      does not use, are not formed; the list read-backs keep what
-                                      the workspace's last tomography call with lists left */
+                                      does not use, are not formed; the read-backs and the counts
+                                      of vg_query keep describing the workspace's last tomography
+                                      call with lists, whatever the beam of this one */
 #define VG_FLAG_SPLAT 16u          /* the 3DGS comparison mode (Sec. 3.2, Eq. 5-7) in the same
                                       pipeline: the density input holds the peak opacity o and
                                       alpha = min(o G'(p), alpha_max), G' the 2D Gaussian with

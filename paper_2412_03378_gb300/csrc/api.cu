@@ -1112,7 +1112,19 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
         const long long items = (long long)nb * N;
         if (items >= 0xFFFFFFFFLL) return fail(ws, VG_ERR_INVALID_ARG, "angles x Gaussians per batch must be < 2^32");
         const long long n_tiles = (long long)nb * tpv;
-        VG_TRY(reserve_items(ws, items));
+        // the backward's item order: by the tile of the footprint's centre (the last key: no footprint), once a
+        // view's weights no longer fit one SM's L1
+        const bool by_home = backward && (long long)beam->det_h * tomo_pitch(beam->det_w) * 4 > kTomoL1Image;
+        if (lists) {
+            VG_TRY(reserve_items(ws, items));
+        } else {   // what the gradient uses; the buffers that the read-backs describe stay as they are
+            VG_TRY(ensure(ws, ws->rec, (size_t)items * kRecF4, "records"));
+            VG_TRY(ensure(ws, ws->count, (size_t)items, "tile counts"));
+            for (int k = 0; k < 2 && by_home; ++k) {
+                VG_TRY(ensure(ws, ws->skey[k], (size_t)items, "sort keys"));
+                VG_TRY(ensure(ws, ws->sval[k], (size_t)items, "sort values"));
+            }
+        }
         VG_TRY(reserve_sort_scratch(ws, items));
         std::vector<ViewInfo> vh((size_t)nb);
         for (int v = 0; v < nb; ++v) {
@@ -1130,20 +1142,17 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
             VG_TRY(ensure(ws, ws->views, vh.size(), "views"));
             VG_CUDA(ws, cudaMemcpyAsync(ws->views.p, vh.data(), vh.size() * sizeof(ViewInfo), cudaMemcpyHostToDevice, st));
         }
-        // the backward's item order: by the tile of the footprint's centre (the last key: no footprint), once a
-        // view's weights no longer fit one SM's L1
-        const bool by_home = backward && (long long)beam->det_h * tomo_pitch(beam->det_w) * 4 > kTomoL1Image;
         uint32_t *home = ws->skey[0].p, *order = nullptr;
         if (items > 0) {
             ProfScope ps(ws, ST_PRE, st);
-            VG_CUDA(ws, cudaMemsetAsync(ws->depth.p, 0xFF, sizeof(uint32_t) * (size_t)items, st));
+            if (lists) VG_CUDA(ws, cudaMemsetAsync(ws->depth.p, 0xFF, sizeof(uint32_t) * (size_t)items, st));
             VG_CUDA(ws, launch_tomo_preprocess(ws->g, ws->tomo_cs.p + 2 * (size_t)a0, nb, beam->det_w, beam->det_h,
                                                beam->pitch_u, beam->pitch_v, beam->u0, beam->v0, opts->tau_cut,
-                                               ws->rec.p, ws->count.p, ws->rect.p, by_home ? home : nullptr, st,
-                                               &ws->launches));
+                                               ws->rec.p, ws->count.p, lists ? ws->rect.p : nullptr,
+                                               by_home ? home : nullptr, st, &ws->launches));
         }
-        long long total = ws->n_inst;
         if (lists) {
+            long long total = 0;
             {
                 ProfScope ps(ws, ST_SCAN, st);
                 VG_CUDA(ws, launch_scan_gather(ws->count.p, nullptr, ws->offsets.p, items, ws->scan_tmp.p,
@@ -1169,6 +1178,11 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
                 ProfScope ps(ws, ST_RANGES, st);
                 VG_CUDA(ws, launch_ranges(ws->inst_key, total, nullptr, ws->ranges.p, n_tiles, false, st, &ws->launches));
             }
+            ws->n_items = items;
+            ws->n_tiles = n_tiles;
+            ws->n_inst = total;
+            ws->n_views = nb;
+            ws->n_pixels = (long long)nb * det_px;
         }
         float *proj_b = proj + (size_t)a0 * det_px;
         if (!proj_given) {
@@ -1197,11 +1211,6 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
                                           beam->pitch_v, beam->u0, beam->v0, ws->grad.p, dmu, dscale, dquat, dkappa,
                                           st, &ws->launches));
         }
-        ws->n_items = items;
-        ws->n_tiles = n_tiles;
-        ws->n_inst = total;
-        ws->n_views = nb;
-        ws->n_pixels = (long long)nb * det_px;
     }
     ws->stage = 0;
     if (lists) ws->tomo_read = true;

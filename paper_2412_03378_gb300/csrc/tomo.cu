@@ -122,7 +122,7 @@ k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det
             }
         }
         count[it] = cnt;
-        rect[it] = rc;
+        if (rect) rect[it] = rc;
         if (home) home[it] = hm;   // the tile of the rectangle's centre
     }
 }
