@@ -340,12 +340,13 @@ cudaError_t launch_tomo_weights(const float *proj, const float *dL, const float 
 // weight tau the partials of ln tau = ln A - |y|^2 / 2 follow from sum G, G y and G y y^T in the
 // whitened coordinates, where they are well conditioned for any elongation.  A lane owns eight pixel
 // columns (two 16-byte loads per row, requested a row ahead; columns left or right of the rectangle sit
-// at y0 = kFar, where tau is 0) and every LY-th row, so that a row's shared terms and sums serve
+// at y0 = kFar, where tau is 0; only an item whose sums come out not finite is summed again with their weights masked,
+// which costs 1.6% here against 7% for masking every row) and every LY-th row, so that a row's shared terms and sums serve
 // eight pixels; 1, 2 or 4 lanes stand side by side, as the rectangle is wide.  The loop is bound by the
 // FMA pipe (a packed instruction holds it for two cycles): about 65 cycles per row of eight pixels.
 // order (may be NULL: item order) lists the items by the tile of their centre and a CTA takes a run of
 // them, so that its warps read the same part of the weights from L1; a warp's items are requested
-// together (one per lane) before the first is summed.  On the workload above 23.4 ms (item sort and chain
+// together (one per lane) before the first is summed.  On the workload above 23.7 ms (item sort and chain
 // included) against 62.4 ms for one reduction per (tile, Gaussian) in tile order; without the home order
 // 27 ms, at 1 / 2 / 8 / 32 items a warp 26.9 / 26.1 / 23.6 / 23.4 ms, at 2 or 4 CTAs per SM 25-29 ms.
 constexpr int kTomoBwdWarps = 8, kTomoBwdCtas = 3;   // warps per CTA, CTAs per SM
@@ -387,54 +388,70 @@ k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch
         const int lxb = min(o1 - o0, 2);   // log2 of the lanes side by side
         const int lx = lane & ((1 << lxb) - 1), ly = lane >> lxb, LY = 32 >> lxb;
         const float LYf = (float)LY;
-        float m0 = 0.0f, n0 = 0.0f, n1 = 0.0f, m01 = 0.0f, m11 = 0.0f;
-        F2 m00 = f2_dup(0.0f);
-        for (int o = o0 + lx; o <= o1; o += 1 << lxb) {
-            F2 b[4];
+        float m0, n0, n1, m01, m11;
+        F2 m00;
+        auto sum_up = [&](auto mask_columns) {
+            m0 = n0 = n1 = m01 = m11 = 0.0f;
+            m00 = f2_dup(0.0f);
+            for (int o = o0 + lx; o <= o1; o += 1 << lxb) {
+                F2 b[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int x = 8 * o + 2 * c;
-                b[c] = f2_pack((x < rx0 || x > rx1) ? kFar : r0.z * ((float)x - r0.x),
-                               (x + 1 < rx0 || x + 1 > rx1) ? kFar : r0.z * ((float)(x + 1) - r0.x));
-            }
-            const float4 *src = reinterpret_cast<const float4 *>(img + (long long)(ry0 + ly) * pitch + 8 * o);
-            float yf = (float)(ry0 + ly);
-            float4 na = make_float4(0.0f, 0.0f, 0.0f, 0.0f), nb = na;
-            if (ry0 + ly <= ry1) {
-                na = __ldg(src);
-                nb = __ldg(src + 1);
-            }
-            for (int y = ry0 + ly; y <= ry1; y += LY) {
-                const F2 g[4] = {f2_pack(na.x, na.y), f2_pack(na.z, na.w), f2_pack(nb.x, nb.y), f2_pack(nb.z, nb.w)};
-                src += (size_t)(LY * (pitch >> 2));
-                if (y + LY <= ry1) {
+                for (int c = 0; c < 4; ++c) {
+                    const int x = 8 * o + 2 * c;
+                    b[c] = f2_pack((x < rx0 || x > rx1) ? kFar : r0.z * ((float)x - r0.x),
+                                   (x + 1 < rx0 || x + 1 > rx1) ? kFar : r0.z * ((float)(x + 1) - r0.x));
+                }
+                const float4 *src = reinterpret_cast<const float4 *>(img + (long long)(ry0 + ly) * pitch + 8 * o);
+                float yf = (float)(ry0 + ly);
+                float4 na = make_float4(0.0f, 0.0f, 0.0f, 0.0f), nb = na;
+                if (ry0 + ly <= ry1) {
                     na = __ldg(src);
                     nb = __ldg(src + 1);
                 }
-                const float dy = yf - r0.y;
-                yf += LYf;
-                const float v = r1.x * dy;
-                const F2 wd = f2_dup(r0.w * dy), Ld = f2_dup(fmaf(v, v, -r1.y));
-                F2 G[4], u[4];
+                for (int y = ry0 + ly; y <= ry1; y += LY) {
+                    F2 g[4] = {f2_pack(na.x, na.y), f2_pack(na.z, na.w), f2_pack(nb.x, nb.y), f2_pack(nb.z, nb.w)};
+                    if constexpr (mask_columns) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const F2 yc = f2_add(b[c], wd);
-                    float a0, a1;
-                    f2_unpack(f2_fma(yc, yc, Ld), a0, a1);
-                    G[c] = f2_mul(g[c], f2_pack(ex2_approx(-a0), ex2_approx(-a1)));
-                    u[c] = f2_mul(G[c], yc);
-                    m00 = f2_fma(u[c], yc, m00);
+                        for (int c = 0; c < 4; ++c) {
+                            const int x = 8 * o + 2 * c;
+                            float w0, w1;
+                            f2_unpack(g[c], w0, w1);
+                            g[c] = f2_pack(x < rx0 || x > rx1 ? 0.0f : w0, x + 1 < rx0 || x + 1 > rx1 ? 0.0f : w1);
+                        }
+                    }
+                    src += (size_t)(LY * (pitch >> 2));
+                    if (y + LY <= ry1) {
+                        na = __ldg(src);
+                        nb = __ldg(src + 1);
+                    }
+                    const float dy = yf - r0.y;
+                    yf += LYf;
+                    const float v = r1.x * dy;
+                    const F2 wd = f2_dup(r0.w * dy), Ld = f2_dup(fmaf(v, v, -r1.y));
+                    F2 G[4], u[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const F2 yc = f2_add(b[c], wd);
+                        float a0, a1;
+                        f2_unpack(f2_fma(yc, yc, Ld), a0, a1);
+                        G[c] = f2_mul(g[c], f2_pack(ex2_approx(-a0), ex2_approx(-a1)));
+                        u[c] = f2_mul(G[c], yc);
+                        m00 = f2_fma(u[c], yc, m00);
+                    }
+                    const float Gs = f2_sum(f2_add(f2_add(G[0], G[1]), f2_add(G[2], G[3])));
+                    const float us = f2_sum(f2_add(f2_add(u[0], u[1]), f2_add(u[2], u[3])));
+                    const float tv = v * Gs;
+                    m0 += Gs;
+                    n0 += us;
+                    n1 += tv;
+                    m01 = fmaf(v, us, m01);
+                    m11 = fmaf(v, tv, m11);
                 }
-                const float Gs = f2_sum(f2_add(f2_add(G[0], G[1]), f2_add(G[2], G[3])));
-                const float us = f2_sum(f2_add(f2_add(u[0], u[1]), f2_add(u[2], u[3])));
-                const float tv = v * Gs;
-                m0 += Gs;
-                n0 += us;
-                n1 += tv;
-                m01 = fmaf(v, us, m01);
-                m11 = fmaf(v, tv, m11);
             }
-        }
+        };
+        sum_up(std::false_type());
+        // a weight that is not finite makes 0 x weight of a column outside the rectangle NaN: sum again without them
+        if (__any_sync(0xffffffffu, !isfinite(m0))) sum_up(std::true_type());
         float v[kTomoGradN] = {m0, n0, n1, f2_sum(m00), m01, m11, 0.0f, 0.0f};
         const int k = warp_reduce_scatter_part<kTomoGradN, 3>(v, lane);
         v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
