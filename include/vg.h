@@ -154,6 +154,13 @@ typedef struct {
                                       does not use, are not formed; the read-backs and the counts
                                       of vg_query keep describing the workspace's last tomography
                                       call with lists, whatever the beam of this one */
+#define VG_FLAG_PROJ_CHECKED 128u  /* vg_project_tomo with dL_dproj: proj holds the projection that the
+                                      workspace's last call (vg_project_tomo, no other since) wrote, or
+                                      a copy.  Its records, if still there, are compared bit for bit with
+                                      the present ones (one synchronisation): while they are the same
+                                      neither the projection nor the lists are formed again, whatever
+                                      was written to the Gaussians in between; else both are, and proj
+                                      is overwritten.  Takes the place of VG_FLAG_PROJ_GIVEN */
 #define VG_FLAG_SPLAT 16u          /* the 3DGS comparison mode (Sec. 3.2, Eq. 5-7) in the same
                                       pipeline: the density input holds the peak opacity o and
                                       alpha = min(o G'(p), alpha_max), G' the 2D Gaussian with

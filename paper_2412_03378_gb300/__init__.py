@@ -29,6 +29,7 @@ FLAG_DENSITY_THETA = 8
 FLAG_SPLAT = 16
 FLAG_PROJ_GIVEN = 32
 FLAG_NO_LISTS = 64
+FLAG_PROJ_CHECKED = 128
 # stage names of the event profiler, in the bit order of vg_profile_stages
 STAGES = ("preprocess", "depth_sort", "scan", "duplicate", "tile_sort", "ranges", "render_fwd", "render_bwd",
           "chain", "l2_loss", "tomo_fwd", "tomo_bwd", "voxel_eval", "ray_march")
@@ -495,9 +496,9 @@ class _RenderFn(torch.autograd.Function):
 
 
 class _TomoFn(torch.autograd.Function):
-    """proj = exp(-sum tau) of a parallel beam (vg_project_tomo); the backward calls it again with
-    dL/dproj.  It hands over its own copy of the projection, and leaves the workspace's tile lists
-    alone while they are the forward's; parameters written to in between are projected anew."""
+    """proj = exp(-sum tau) of a parallel beam (vg_project_tomo); the backward calls it again with dL/dproj.  It hands
+    over its own copy of the projection, which the library takes while the records it was made of are still in the
+    workspace and unchanged, and projects anew otherwise: a gradient is always that of the parameters as they are."""
 
     @staticmethod
     def forward(ctx, ws, beam, opts, keep, mu, scale, quat, kappa):
@@ -506,13 +507,9 @@ class _TomoFn(torch.autograd.Function):
         proj = torch.empty((len(beam.angles), int(beam.det_h), int(beam.det_w)), device=mu.device,
                            dtype=torch.float32)
         ws.project_tomo(g, beam, opts, proj)
-        if not keep:   # no backward can come (and a tensor of inference mode has no version counter)
+        if not keep:   # no backward can come
             return proj
         ctx.ws, ctx.beam, ctx.opts, ctx.g, ctx.gen = ws, beam, opts, g, ws.generation
-        ctx.seen = [t._version for t in (g.mu, g.scale, g.quat, g.kappa)]
-        ctx.angles = [float(a) for a in beam.angles]
-        ctx.geometry = (int(beam.det_w), int(beam.det_h), float(beam.pitch_u), float(beam.pitch_v), float(beam.u0),
-                        float(beam.v0), opts.tau_cut, opts.flags)
         try:
             ctx.proj = proj.clone()
         except torch.OutOfMemoryError:
@@ -521,22 +518,16 @@ class _TomoFn(torch.autograd.Function):
 
     @staticmethod
     def backward(ctx, g_proj):
-        g, beam, opts = ctx.g, ctx.beam, ctx.opts
+        g, ws = ctx.g, ctx.ws
         params = (g.mu, g.scale, g.quat, g.kappa)
         grads = _grad_buffers(g, *params)
-        flags = opts.flags | FLAG_GRAD_ZERO
-        same = ctx.proj is not None and ctx.seen == [t._version for t in params] and \
-            ctx.geometry == (int(beam.det_w), int(beam.det_h), float(beam.pitch_u), float(beam.pitch_v), float(beam.u0),
-                             float(beam.v0), opts.tau_cut, opts.flags) and \
-            ctx.angles == [float(a) for a in beam.angles]
-        if same:
-            proj = ctx.proj
-            flags |= FLAG_PROJ_GIVEN | (FLAG_NO_LISTS if ctx.ws.generation == ctx.gen else 0)
-        else:
-            proj = torch.empty_like(g_proj, dtype=torch.float32)
-        o = copy.copy(opts)
-        o.flags = flags
-        ctx.ws.project_tomo(g, beam, o, proj, g_proj.contiguous().float(), *grads)
+        own = ctx.proj is not None and ws.generation == ctx.gen
+        proj = ctx.proj if own else torch.empty_like(g_proj, dtype=torch.float32)
+        o = copy.copy(ctx.opts)
+        o.flags = o.flags & ~FLAG_PROJ_GIVEN | FLAG_GRAD_ZERO | (FLAG_PROJ_CHECKED if own else 0)
+        ws.project_tomo(g, ctx.beam, o, proj, g_proj.contiguous().float(), *grads)
+        if own:   # the workspace still holds this forward's records, or those of the parameters that proj was formed of
+            ctx.gen = ws.generation
         return (None, None, None, None) + tuple(d.to(t.dtype) for d, t in zip(grads, params))
 
 

@@ -69,6 +69,8 @@ struct vg_workspace {
     uint32_t *tile_order = nullptr;       // longest-first tile order of the last bin_sort
     bool treplay_clear = false;           // treplay is zero since the last binning
     bool replay_known = false;            // treplay holds the last forward's replay lengths
+    bool tomo_rec = false;                // rec and count are those of the last tomography call with lists, of
+    int tomo_n = 0, tomo_a = 0, tomo_w = 0, tomo_h = 0;   // so many Gaussians, angles and detector pixels (one batch)
     DBuf<uint32_t> treplay, tord_bwd;     // per-tile replay lengths and their order
     int ppt_fwd = 2, ppt_bwd = 1;         // pixels per thread of the blend kernels
     int tuned_fwd = 0, tuned_bwd = 0;     // vg_autotune's choice (0: none yet)
@@ -330,6 +332,7 @@ static vg_status reserve_sort_scratch(vg_workspace *ws, long long n) {
 
 static unsigned long long *total64_ptr(vg_workspace *ws) { return ws->counters.p + 6; }
 static uint32_t *lookback_err_ptr(vg_workspace *ws) { return (uint32_t *)(ws->counters.p + 7); }
+static uint32_t *tomo_changed_ptr(vg_workspace *ws) { return lookback_err_ptr(ws) + 1; }   // h_total[3] when read
 // The backward's tile order: by the replay lengths the last forward measured (longest first), else the binning's.
 static cudaError_t bwd_order(vg_workspace *ws, cudaStream_t st, const int **order) {
     *order = (const int *)ws->tile_order;
@@ -392,6 +395,7 @@ vg_status vg_workspace_reserve(vg_workspace *ws, int64_t n_items, int64_t n_inst
         return fail(ws, VG_ERR_INVALID_ARG, "negative reservation");
     const unsigned flags = ws->opts.flags;
     ws->opts.flags &= ~VG_FLAG_FIXED_CAPACITY;
+    ws->tomo_rec = false;   // the buffers may be replaced
     vg_status s = reserve_items(ws, n_items);
     if (s == VG_OK) s = reserve_sort_scratch(ws, n_items);
     if (s == VG_OK) s = reserve_instances(ws, n_instances);
@@ -488,7 +492,7 @@ static vg_status preprocess_impl(vg_workspace *ws, const vg_gaussians *g, const 
     ws->g.softplus_beta = opts->softplus_beta;
     ws->g.splat = splat ? 1 : 0;
     ws->g.splat_dil = splat ? opts->splat_dilation : 0.0f;
-    ws->tomo_read = false;
+    ws->tomo_read = ws->tomo_rec = false;
     VG_TRY(reserve_items(ws, n_items));
     VG_TRY(upload_views(ws, vh, tv, st));
     ws->n_views = n_views;
@@ -534,6 +538,7 @@ static vg_status upload_views(vg_workspace *ws, const std::vector<ViewInfo> &vh,
 
 // Per-item records, depth keys and tile footprints of the workspace's Gaussians and views.
 static vg_status run_preprocess(vg_workspace *ws, cudaStream_t st) {
+    ws->tomo_rec = false;
     VG_CUDA(ws, cudaMemsetAsync(ws->counters.p, 0, sizeof(unsigned long long), st));
     if (ws->n_items > 0) {
         ProfScope ps(ws, ST_PRE, st);
@@ -896,7 +901,7 @@ vg_status vg_query_density(vg_workspace *ws, const vg_gaussians *g, const vg_gri
     ws->g.sh = nullptr;
     ws->g.density_theta = (opts->flags & VG_FLAG_DENSITY_THETA) ? 1 : 0;
     ws->stage = 0;   // the render state of this workspace is overwritten below
-    ws->views_valid = false;
+    ws->views_valid = ws->tomo_rec = false;
     VG_TRY(reserve_items(ws, n));
     VG_TRY(reserve_sort_scratch(ws, n));
     VG_TRY(ensure(ws, ws->vbox, (size_t)n * 2, "voxel boxes"));
@@ -1065,8 +1070,8 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
                            float *dmu, float *dscale, float *dquat, float *dkappa, cudaStream_t st) {
     const bool fused = target != nullptr;
     const bool backward = dL_dproj != nullptr || fused;
-    const bool proj_given = dL_dproj && !fused && (opts && (opts->flags & VG_FLAG_PROJ_GIVEN));
-    const bool lists = !proj_given || !(opts->flags & VG_FLAG_NO_LISTS);   // the projection alone needs them
+    bool proj_given = dL_dproj && !fused && (opts && (opts->flags & VG_FLAG_PROJ_GIVEN));
+    bool lists = !proj_given || !(opts->flags & VG_FLAG_NO_LISTS);   // the projection alone needs them
     VG_TRY(check_gauss(ws, g, false));
     if (!beam || beam->n_angles < 1 || !beam->angles || beam->det_w <= 0 || beam->det_h <= 0 ||
         !finite_pos(beam->pitch_u) || !finite_pos(beam->pitch_v) || !std::isfinite(beam->u0) ||
@@ -1088,6 +1093,11 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
     ws->g.density_theta = (opts->flags & VG_FLAG_DENSITY_THETA) ? 1 : 0;
     ws->stage = 0;   // the render state of this workspace is overwritten below
     ws->views_valid = false;
+    // the projection of records that are still here: whether they changed is seen where they are formed anew
+    const bool check = dL_dproj && !fused && (opts->flags & VG_FLAG_PROJ_CHECKED) && ws->tomo_rec && ws->tomo_n == N &&
+                       ws->tomo_a == A && ws->tomo_w == beam->det_w && ws->tomo_h == beam->det_h && N > 0;
+    ws->tomo_rec = false;
+    if (check) proj_given = lists = true;
     std::vector<float> cs(2 * (size_t)A);
     for (int a = 0; a < A; ++a) {
         if (!std::isfinite(beam->angles[a])) return fail(ws, VG_ERR_INVALID_ARG, "non-finite beam angle");
@@ -1126,22 +1136,6 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
             }
         }
         VG_TRY(reserve_sort_scratch(ws, items));
-        std::vector<ViewInfo> vh((size_t)nb);
-        for (int v = 0; v < nb; ++v) {
-            memset(&vh[v], 0, sizeof(ViewInfo));
-            vh[v].W = beam->det_w;
-            vh[v].H = beam->det_h;
-            vh[v].tw = kTile;
-            vh[v].th = kTile;
-            vh[v].tiles_x = tiles_x;
-            vh[v].tiles_y = tiles_y;
-            vh[v].tile_base = (int)(v * tpv);
-            vh[v].pix_base = (long long)v * det_px;
-        }
-        if (lists) {
-            VG_TRY(ensure(ws, ws->views, vh.size(), "views"));
-            VG_CUDA(ws, cudaMemcpyAsync(ws->views.p, vh.data(), vh.size() * sizeof(ViewInfo), cudaMemcpyHostToDevice, st));
-        }
         uint32_t *home = ws->skey[0].p, *order = nullptr;
         if (items > 0) {
             ProfScope ps(ws, ST_PRE, st);
@@ -1149,10 +1143,32 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
             VG_CUDA(ws, launch_tomo_preprocess(ws->g, ws->tomo_cs.p + 2 * (size_t)a0, nb, beam->det_w, beam->det_h,
                                                beam->pitch_u, beam->pitch_v, beam->u0, beam->v0, opts->tau_cut,
                                                ws->rec.p, ws->count.p, lists ? ws->rect.p : nullptr,
-                                               by_home ? home : nullptr, st, &ws->launches));
+                                               by_home ? home : nullptr, check ? tomo_changed_ptr(ws) : nullptr, st,
+                                               &ws->launches));
+        }
+        if (check) {
+            long long unused;
+            VG_TRY(read_total(ws, st, &unused));
+            proj_given = ws->h_total[3] == 0;
+            lists = !proj_given;
+            if (lists) VG_CUDA(ws, cudaMemsetAsync(tomo_changed_ptr(ws), 0, sizeof(uint32_t), st));
         }
         if (lists) {
             long long total = 0;
+            std::vector<ViewInfo> vh((size_t)nb);
+            for (int v = 0; v < nb; ++v) {
+                memset(&vh[v], 0, sizeof(ViewInfo));
+                vh[v].W = beam->det_w;
+                vh[v].H = beam->det_h;
+                vh[v].tw = kTile;
+                vh[v].th = kTile;
+                vh[v].tiles_x = tiles_x;
+                vh[v].tiles_y = tiles_y;
+                vh[v].tile_base = (int)(v * tpv);
+                vh[v].pix_base = (long long)v * det_px;
+            }
+            VG_TRY(ensure(ws, ws->views, vh.size(), "views"));
+            VG_CUDA(ws, cudaMemcpyAsync(ws->views.p, vh.data(), vh.size() * sizeof(ViewInfo), cudaMemcpyHostToDevice, st));
             {
                 ProfScope ps(ws, ST_SCAN, st);
                 VG_CUDA(ws, launch_scan_gather(ws->count.p, nullptr, ws->offsets.p, items, ws->scan_tmp.p,
@@ -1214,6 +1230,8 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
     }
     ws->stage = 0;
     if (lists) ws->tomo_read = true;
+    ws->tomo_rec = (lists || check) && batch >= A;
+    ws->tomo_n = N, ws->tomo_a = A, ws->tomo_w = beam->det_w, ws->tomo_h = beam->det_h;
     return VG_OK;
 }
 

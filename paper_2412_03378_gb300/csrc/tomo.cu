@@ -71,12 +71,18 @@ __device__ __forceinline__ void tomo_geom(const float mu[3], const float s[3], c
     G.jmu = (mu[2] - v0) / pv - 0.5f;
 }
 
+__device__ __forceinline__ bool same_bits(const float4 &a, const float4 &b) {
+    return __float_as_uint(a.x) == __float_as_uint(b.x) && __float_as_uint(a.y) == __float_as_uint(b.y) &&
+           __float_as_uint(a.z) == __float_as_uint(b.z) && __float_as_uint(a.w) == __float_as_uint(b.w);
+}
+
 // ---------------------------------------------------------------------------- preprocess
+// changed (may be NULL): set where a record or a count differs from what the buffers hold
 template <typename RT>
 __global__ void __launch_bounds__(256)
 k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det_w, int det_h, float pu, float pv,
                   float u0, float v0, float tau_cut, float4 *__restrict__ rec, uint32_t *__restrict__ count,
-                  short4 *__restrict__ rect, uint32_t *__restrict__ home) {
+                  short4 *__restrict__ rect, uint32_t *__restrict__ home, uint32_t *__restrict__ changed) {
     pdl_entry();
     const long long n_items = (long long)g.n * n_angles;
     const int tiles_x = (det_w + kTile - 1) / kTile, tiles_y = (det_h + kTile - 1) / kTile;
@@ -116,11 +122,15 @@ k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det
                 tomo_geom(mu, s, Rq, ct, st, pu, pv, u0, v0, G);
                 const float lnA2 = log2f(kap) + kLog2Sqrt2Pi - log2f(G.n);
                 // the pixel rectangle (< 32768 on both axes) rides in the record's last two words
-                rec[2 * it] = make_float4(G.imu, G.jmu, G.l00 * kYScale, G.l10 * kYScale);
-                rec[2 * it + 1] = make_float4(G.l11 * kYScale, lnA2, __uint_as_float((unsigned)ix0 | (unsigned)ix1 << 16),
+                const float4 q0 = make_float4(G.imu, G.jmu, G.l00 * kYScale, G.l10 * kYScale);
+                const float4 q1 = make_float4(G.l11 * kYScale, lnA2, __uint_as_float((unsigned)ix0 | (unsigned)ix1 << 16),
                                               __uint_as_float((unsigned)iy0 | (unsigned)iy1 << 16));
+                if (changed && !(same_bits(rec[2 * it], q0) && same_bits(rec[2 * it + 1], q1))) *changed = 1u;
+                rec[2 * it] = q0;
+                rec[2 * it + 1] = q1;
             }
         }
+        if (changed && count[it] != cnt) *changed = 1u;
         count[it] = cnt;
         if (rect) rect[it] = rc;
         if (home) home[it] = hm;   // the tile of the rectangle's centre
@@ -129,7 +139,7 @@ k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det
 
 cudaError_t launch_tomo_preprocess(const GaussIn &g, const float *cs_d, int n_angles, int det_w, int det_h,
                                    float pitch_u, float pitch_v, float u0, float v0, float tau_cut, float4 *rec,
-                                   uint32_t *count, short4 *rect, uint32_t *home, cudaStream_t st,
+                                   uint32_t *count, short4 *rect, uint32_t *home, uint32_t *changed, cudaStream_t st,
                                    long long *launches) {
     const long long n_items = (long long)g.n * n_angles;
     long long b = (n_items + 255) / 256;
@@ -138,13 +148,13 @@ cudaError_t launch_tomo_preprocess(const GaussIn &g, const float *cs_d, int n_an
     *launches += 1;
     if (g.rec_dtype == VG_BF16)
         pdl_launch(k_tomo_preprocess<__nv_bfloat16>, (unsigned)b, 256, 0, st, g, cs_d, n_angles, det_w, det_h, pitch_u, pitch_v,
-                                                                      u0, v0, tau_cut, rec, count, rect, home);
+                                                                      u0, v0, tau_cut, rec, count, rect, home, changed);
     else if (g.rec_dtype == VG_F16)
         pdl_launch(k_tomo_preprocess<__half>, (unsigned)b, 256, 0, st, g, cs_d, n_angles, det_w, det_h, pitch_u, pitch_v, u0,
-                                                               v0, tau_cut, rec, count, rect, home);
+                                                               v0, tau_cut, rec, count, rect, home, changed);
     else
         pdl_launch(k_tomo_preprocess<float>, (unsigned)b, 256, 0, st, g, cs_d, n_angles, det_w, det_h, pitch_u, pitch_v, u0,
-                                                              v0, tau_cut, rec, count, rect, home);
+                                                              v0, tau_cut, rec, count, rect, home, changed);
     return cudaGetLastError();
 }
 

@@ -159,7 +159,7 @@ cudaError_t launch_preprocess(const GaussIn &g, const ViewInfo *views_d, int n_v
 cudaError_t launch_tomo_preprocess(const GaussIn &g, const float *cs_d /* [A][2] cos, sin */, int n_angles,
                                    int det_w, int det_h, float pitch_u, float pitch_v, float u0, float v0,
                                    float tau_cut, float4 *rec, uint32_t *count, short4 *rect, uint32_t *home,
-                                   cudaStream_t st, long long *launches);
+                                   uint32_t *changed, cudaStream_t st, long long *launches);
 
 // Buffers (16-byte aligned, in 32-bit words) zeroed by one launch.
 struct ClearList {
