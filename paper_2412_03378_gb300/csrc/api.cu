@@ -407,6 +407,8 @@ vg_status vg_workspace_reserve(vg_workspace *ws, int64_t n_items, int64_t n_inst
     if (s == VG_OK) s = ensure(ws, ws->tile_view, (size_t)n_tiles, "tile views");
     if (s == VG_OK) s = ensure(ws, ws->grad, (size_t)n_items * kGradN, "gradient accumulators");
     if (s == VG_OK) s = ensure(ws, ws->tord, (size_t)n_tiles, "tile order");
+    // a tomography's weights in rows padded to 8 pixels: they fit its 16 x 16 tiles
+    if (s == VG_OK) s = ensure(ws, ws->tomo_dl, (size_t)std::min(8 * n_pixels, 256 * n_tiles), "pixel weights");
     ws->opts.flags = flags;
     return s;
 }
@@ -1098,6 +1100,19 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
                        ws->tomo_a == A && ws->tomo_w == beam->det_w && ws->tomo_h == beam->det_h && N > 0;
     ws->tomo_rec = false;
     if (check) proj_given = lists = true;
+    // angles are processed in batches of at most ~4M (angle, Gaussian) items
+    const long long budget = 1LL << 22;
+    int batch = N > 0 ? (int)std::max<long long>(1, std::min<long long>(A, budget / N)) : A;
+    while ((long long)batch * tpv >= (1LL << 30) && batch > 1) batch /= 2;
+    // the pixels' weights of the backward, an image of padded rows; without it (a fixed-capacity workspace whose buffer is
+    // smaller, no memory) the backward forms them from proj where it uses them
+    bool weights = false;
+    if (backward) {
+        const size_t words = (size_t)batch * beam->det_h * tomo_pitch(beam->det_w);
+        if (ws->tomo_dl.n >= words || !ws->tomo_dl.p || !(opts->flags & VG_FLAG_FIXED_CAPACITY))
+            weights = ensure(ws, ws->tomo_dl, words, "pixel weights") == VG_OK;
+        if (!weights) ws->err.clear();
+    }
     std::vector<float> cs(2 * (size_t)A);
     for (int a = 0; a < A; ++a) {
         if (!std::isfinite(beam->angles[a])) return fail(ws, VG_ERR_INVALID_ARG, "non-finite beam angle");
@@ -1113,10 +1128,6 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
         VG_CUDA(ws, cudaMemsetAsync(dquat, 0, (size_t)N * 4 * sizeof(float), st));
         VG_CUDA(ws, cudaMemsetAsync(dkappa, 0, (size_t)N * sizeof(float), st));
     }
-    // angles are processed in batches of at most ~4M (angle, Gaussian) items
-    const long long budget = 1LL << 22;
-    int batch = N > 0 ? (int)std::max<long long>(1, std::min<long long>(A, budget / N)) : A;
-    while ((long long)batch * tpv >= (1LL << 30) && batch > 1) batch /= 2;
     for (int a0 = 0; a0 < A; a0 += batch) {
         const int nb = std::min(batch, A - a0);
         const long long items = (long long)nb * N;
@@ -1207,11 +1218,12 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
                                         ws->inst_item, ws->rec.p, proj_b, st, &ws->launches));
         }
         const float *dl_b = dL_dproj ? dL_dproj + (size_t)a0 * det_px : nullptr;
-        if (backward) {   // the pixels' weights dL/dtau and, fused, the batch's share of the loss
-            VG_TRY(ensure(ws, ws->tomo_dl, (size_t)nb * beam->det_h * tomo_pitch(beam->det_w), "pixel weights"));
+        const float *target_b = fused ? target + (size_t)a0 * det_px : nullptr;
+        float *weights_b = weights ? ws->tomo_dl.p : nullptr;
+        if (backward && (weights || fused)) {   // the pixels' weights dL/dtau and, fused, the batch's share of the loss
             ProfScope ps(ws, ST_LOSS, st);
-            VG_CUDA(ws, launch_tomo_weights(proj_b, dl_b, fused ? target + (size_t)a0 * det_px : nullptr, scale, loss, nb,
-                                            beam->det_w, beam->det_h, ws->tomo_dl.p, st, &ws->launches));
+            VG_CUDA(ws, launch_tomo_weights(proj_b, dl_b, target_b, scale, loss, nb, beam->det_w, beam->det_h, weights_b, st,
+                                            &ws->launches));
         }
         if (backward && items > 0) {
             VG_TRY(ensure(ws, ws->grad, (size_t)items * 8, "gradient accumulators"));
@@ -1221,8 +1233,8 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
                 VG_CUDA(ws, launch_radix_sort(home, nullptr, ws->skey[1].p, ws->sval[1].p, ws->skey[0].p, ws->sval[0].p, items,
                                               nullptr, bits_for(n_tiles + 1), ws->hist.p, lookback_err_ptr(ws), false, &home, &order, st,
                                               &ws->launches));
-            VG_CUDA(ws, launch_tomo_bwd(items, N, beam->det_w, beam->det_h, order, ws->count.p, ws->rec.p, ws->tomo_dl.p,
-                                        ws->grad.p, st, &ws->launches));
+            VG_CUDA(ws, launch_tomo_bwd(items, N, beam->det_w, beam->det_h, order, ws->count.p, ws->rec.p, weights_b, proj_b,
+                                        dl_b, target_b, scale, ws->grad.p, st, &ws->launches));
             VG_CUDA(ws, launch_tomo_chain(ws->g, ws->tomo_cs.p, A, (long long)a0 * N, items, beam->pitch_u,
                                           beam->pitch_v, beam->u0, beam->v0, ws->grad.p, dmu, dscale, dquat, dkappa,
                                           st, &ws->launches));

@@ -317,7 +317,7 @@ k_tomo_weights(const float *__restrict__ proj, const float *__restrict__ dL, con
                     acc = fmaf(e, e, acc);
                 }
             }
-            out[y * pitch + x] = g;
+            if (out) out[y * pitch + x] = g;
         }
     }
     if (dL) return;
@@ -359,13 +359,26 @@ cudaError_t launch_tomo_weights(const float *proj, const float *dL, const float 
 // together (one per lane) before the first is summed.  On the workload above 23.7 ms (item sort and chain
 // included) against 62.4 ms for one reduction per (tile, Gaussian) in tile order; without the home order
 // 27 ms, at 1 / 2 / 8 / 32 items a warp 26.9 / 26.1 / 23.6 / 23.4 ms, at 2 or 4 CTAs per SM 25-29 ms.
+// Where the image of weights cannot be had (a fixed-capacity workspace whose buffer is smaller, no memory) a weight is
+// formed where it is used, by the same operations: one value of proj and one of dL (or target) per pixel and item, unaligned.
+struct TomoDirect {
+    const float *proj, *dL, *target;   // dL NULL: the L2 loss against target
+    float scale;
+    __device__ float operator()(long long i) const {
+        if (dL) return -proj[i] * dL[i];
+        const float e = proj[i] - target[i];
+        return -proj[i] * (2.0f * scale * e);
+    }
+};
+
 constexpr int kTomoBwdWarps = 8, kTomoBwdCtas = 3;   // warps per CTA, CTAs per SM
 constexpr int kTomoBwdItems = 16;                    // items of a warp, at most
 
+template <bool DIRECT>   // pitch: floats from row to row of the weights, or of proj and dL
 __global__ void __launch_bounds__(32 * kTomoBwdWarps, kTomoBwdCtas)
 k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch, const uint32_t *__restrict__ order,
            const uint32_t *__restrict__ count, const float4 *__restrict__ rec, const float *__restrict__ weights,
-           float *__restrict__ acc) {
+           TomoDirect direct, float *__restrict__ acc) {
     pdl_entry();
     const int lane = threadIdx.x & 31;
     const long long at0 = (long long)blockIdx.x * kTomoBwdWarps * per_warp + (threadIdx.x >> 5);
@@ -393,7 +406,8 @@ k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch
         const unsigned rx = __float_as_uint(__shfl_sync(0xffffffffu, my1.z, from));
         const unsigned ry = __float_as_uint(__shfl_sync(0xffffffffu, my1.w, from));
         const int rx0 = (int)(rx & 0xffffu), rx1 = (int)(rx >> 16), ry0 = (int)(ry & 0xffffu), ry1 = (int)(ry >> 16);
-        const float *img = weights + (it / n_per_view) * (long long)det_h * pitch;
+        const long long img0 = (it / n_per_view) * (long long)det_h * pitch;
+        const float *img = weights + img0;
         const int o0 = rx0 >> 3, o1 = rx1 >> 3;
         const int lxb = min(o1 - o0, 2);   // log2 of the lanes side by side
         const int lx = lane & ((1 << lxb) - 1), ly = lane >> lxb, LY = 32 >> lxb;
@@ -414,23 +428,29 @@ k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch
                 const float4 *src = reinterpret_cast<const float4 *>(img + (long long)(ry0 + ly) * pitch + 8 * o);
                 float yf = (float)(ry0 + ly);
                 float4 na = make_float4(0.0f, 0.0f, 0.0f, 0.0f), nb = na;
-                if (ry0 + ly <= ry1) {
+                if (!DIRECT && ry0 + ly <= ry1) {
                     na = __ldg(src);
                     nb = __ldg(src + 1);
                 }
                 for (int y = ry0 + ly; y <= ry1; y += LY) {
                     F2 g[4] = {f2_pack(na.x, na.y), f2_pack(na.z, na.w), f2_pack(nb.x, nb.y), f2_pack(nb.z, nb.w)};
-                    if constexpr (mask_columns) {
+                    if constexpr (DIRECT || mask_columns) {
 #pragma unroll
                         for (int c = 0; c < 4; ++c) {
                             const int x = 8 * o + 2 * c;
+                            const bool in0 = x >= rx0 && x <= rx1, in1 = x + 1 >= rx0 && x + 1 <= rx1;
                             float w0, w1;
                             f2_unpack(g[c], w0, w1);
-                            g[c] = f2_pack(x < rx0 || x > rx1 ? 0.0f : w0, x + 1 < rx0 || x + 1 > rx1 ? 0.0f : w1);
+                            if constexpr (DIRECT) {
+                                const long long i = img0 + (long long)y * pitch + x;
+                                w0 = in0 ? direct(i) : 0.0f;
+                                w1 = in1 ? direct(i + 1) : 0.0f;
+                            }
+                            g[c] = f2_pack(in0 ? w0 : 0.0f, in1 ? w1 : 0.0f);
                         }
                     }
                     src += (size_t)(LY * (pitch >> 2));
-                    if (y + LY <= ry1) {
+                    if (!DIRECT && y + LY <= ry1) {
                         na = __ldg(src);
                         nb = __ldg(src + 1);
                     }
@@ -461,7 +481,7 @@ k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch
         };
         sum_up(std::false_type());
         // a weight that is not finite makes 0 x weight of a column outside the rectangle NaN: sum again without them
-        if (__any_sync(0xffffffffu, !isfinite(m0))) sum_up(std::true_type());
+        if (!DIRECT && __any_sync(0xffffffffu, !isfinite(m0))) sum_up(std::true_type());
         float v[kTomoGradN] = {m0, n0, n1, f2_sum(m00), m01, m11, 0.0f, 0.0f};
         const int k = warp_reduce_scatter_part<kTomoGradN, 3>(v, lane);
         v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
@@ -471,15 +491,21 @@ k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch
 }
 
 cudaError_t launch_tomo_bwd(long long n_items, int n_per_view, int det_w, int det_h, const uint32_t *order,
-                            const uint32_t *count, const float4 *rec, const float *weights, float *acc, cudaStream_t st,
+                            const uint32_t *count, const float4 *rec, const float *weights, const float *proj,
+                            const float *dL, const float *target, float scale, float *acc, cudaStream_t st,
                             long long *launches) {
     if (n_items <= 0) return cudaSuccess;
     // several items a warp while that leaves four CTAs for every resident one
     const long long resident = 152 * kTomoBwdCtas * kTomoBwdWarps;
     const int per = (int)std::max<long long>(1, std::min<long long>(kTomoBwdItems, n_items / (4 * resident)));
     const long long b = (n_items + (long long)kTomoBwdWarps * per - 1) / ((long long)kTomoBwdWarps * per);
-    pdl_launch(k_tomo_bwd, (unsigned)b, 32 * kTomoBwdWarps, 0, st, n_items, per, n_per_view, det_h, tomo_pitch(det_w),
-               order, count, rec, weights, acc);
+    const TomoDirect direct{proj, dL, target, scale};
+    if (weights)
+        pdl_launch(k_tomo_bwd<false>, (unsigned)b, 32 * kTomoBwdWarps, 0, st, n_items, per, n_per_view, det_h, tomo_pitch(det_w),
+                   order, count, rec, weights, direct, acc);
+    else
+        pdl_launch(k_tomo_bwd<true>, (unsigned)b, 32 * kTomoBwdWarps, 0, st, n_items, per, n_per_view, det_h, det_w, order, count,
+                   rec, weights, direct, acc);
     *launches += 1;
     return cudaGetLastError();
 }

@@ -291,16 +291,17 @@ cudaError_t launch_tomo_fwd(const uint2 *ranges, long long n_tiles, int tiles_x,
 
 // The pixel weights of the tomography backward, dL/dtau = -proj dL/dproj, as rows of
 // tomo_pitch(det_w) floats (32-byte aligned, padding zero): from dL, or (dL NULL) from the L2 loss
-// scale sum (proj - target)^2, which is then added to *loss.
+// scale sum (proj - target)^2, which is then added to *loss.  weights NULL: the loss alone.
 inline int tomo_pitch(int det_w) { return (det_w + 7) & ~7; }
 cudaError_t launch_tomo_weights(const float *proj, const float *dL, const float *target, float scale, float *loss,
                                 int n_views, int det_w, int det_h, float *weights, cudaStream_t st,
                                 long long *launches);
 
 // Writes the 8 sums of every item (zeros for one without a footprint) into acc, the items taken in
-// the given order (NULL: their own).
+// the given order (NULL: their own).  weights NULL: formed from proj and dL (or target and scale) where they are used.
 cudaError_t launch_tomo_bwd(long long n_items, int n_per_view, int det_w, int det_h, const uint32_t *order,
-                            const uint32_t *count, const float4 *rec, const float *weights, float *acc, cudaStream_t st,
+                            const uint32_t *count, const float4 *rec, const float *weights, const float *proj,
+                            const float *dL, const float *target, float scale, float *acc, cudaStream_t st,
                             long long *launches);
 
 cudaError_t launch_tomo_chain(const GaussIn &g, const float *cs_d, int n_angles, long long item0, long long n_items,
