@@ -407,6 +407,7 @@ vg_status vg_workspace_reserve(vg_workspace *ws, int64_t n_items, int64_t n_inst
     if (s == VG_OK) s = ensure(ws, ws->tile_view, (size_t)n_tiles, "tile views");
     if (s == VG_OK) s = ensure(ws, ws->grad, (size_t)n_items * kGradN, "gradient accumulators");
     if (s == VG_OK) s = ensure(ws, ws->tord, (size_t)n_tiles, "tile order");
+    if (s == VG_OK) s = ensure(ws, ws->cone_w, (size_t)n_pixels, "pixel weights");   // cone beam
     // a tomography's weights in rows padded to 8 pixels: they fit its 16 x 16 tiles
     if (s == VG_OK) s = ensure(ws, ws->tomo_dl, (size_t)std::min(8 * n_pixels, 256 * n_tiles), "pixel weights");
     ws->opts.flags = flags;
