@@ -81,7 +81,7 @@ typedef struct {
 /* Parallel-beam tomography geometry.  Rotation axis is world z; for angle theta the rays
  * run along d = (cos theta, sin theta, 0) and detector pixel (i, j) sits at
  * u = u0 + (i + 0.5) pitch_u along (-sin theta, cos theta, 0) and v = v0 + (j + 0.5) pitch_v
- * along (0, 0, 1).  `angles` is a HOST array of n_angles radians. */
+ * along (0, 0, 1).  `angles` is a HOST array of n_angles radians; det_w and det_h are 1..65536. */
 typedef struct {
     int32_t n_angles;
     const float *angles;

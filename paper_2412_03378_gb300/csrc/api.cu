@@ -1088,7 +1088,8 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
     if (fused && (!loss || !std::isfinite(scale))) return fail(ws, VG_ERR_INVALID_ARG, "loss is NULL or scale not finite");
     const int A = beam->n_angles, N = g->n;
     const int tiles_x = (beam->det_w + kTile - 1) / kTile, tiles_y = (beam->det_h + kTile - 1) / kTile;
-    if (tiles_x > 32767 || tiles_y > 32767) return fail(ws, VG_ERR_INVALID_ARG, "detector too large");
+    // the records hold a footprint's first and last pixel in 16 bits
+    if (beam->det_w > 65536 || beam->det_h > 65536) return fail(ws, VG_ERR_INVALID_ARG, "detector wider or taller than 65536");
     const long long tpv = (long long)tiles_x * tiles_y;
     const long long det_px = (long long)beam->det_w * beam->det_h;
     ws->opts = *opts;

@@ -121,7 +121,7 @@ k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det
                 TomoGeom G;
                 tomo_geom(mu, s, Rq, ct, st, pu, pv, u0, v0, G);
                 const float lnA2 = log2f(kap) + kLog2Sqrt2Pi - log2f(G.n);
-                // the pixel rectangle (< 32768 on both axes) rides in the record's last two words
+                // the pixel rectangle (< 65536 on both axes) rides in the record's last two words
                 const float4 q0 = make_float4(G.imu, G.jmu, G.l00 * kYScale, G.l10 * kYScale);
                 const float4 q1 = make_float4(G.l11 * kYScale, lnA2, __uint_as_float((unsigned)ix0 | (unsigned)ix1 << 16),
                                               __uint_as_float((unsigned)iy0 | (unsigned)iy1 << 16));
