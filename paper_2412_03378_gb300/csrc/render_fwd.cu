@@ -231,7 +231,7 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                                 // (no pixel of the projection finishes, and footprints end at the image's edge)
                                 bool ok = CONE ? true : (kN == 1 ? ((live >> (c + h * kRow)) & 1u) != 0 : in[i]);
                                 if constexpr (PIXTEST) ok = ok & pixel_in(x0 + c, y0 + h, pr);
-                                if (COUNT) pairs += ok & ((live >> (c + h * kRow)) & 1u);
+                                if (COUNT && kN == 1) pairs += ok & ((live >> (c + h * kRow)) & 1u);
                                 const float t_c = fminf(t[i][c][h], bp.tau_max);
                                 v[i][c][h] = CONE ? ok : ok & (t_c >= bp.tau_skip);   // tau_skip = 0, and t_c is no NaN
                                 t[i][c][h] = v[i][c][h] ? t_c : 0.0f;
@@ -247,6 +247,12 @@ k_render_fwd(const ViewInfo *__restrict__ views, const int *__restrict__ tile_vi
                         const float4 q5 = srec[js[i] * kRF4 + kRF4 - 1];
 #pragma unroll
                         for (int c = 0; c < P / 2; ++c) {
+                            if constexpr (COUNT && kN > 1) {   // (with the pixels that earlier records of the batch finished)
+                                const Rect pr = srect[js[i]];
+#pragma unroll
+                                for (int h = 0; h < 2; ++h)
+                                    pairs += in[i] & pixel_in(x0 + c, y0 + h, pr) & ((live >> (c + h * kRow)) & 1u);
+                            }
                             if (kN > 1 && !CONE) {   // a pixel finished by an earlier record of the batch
                                 float e[2];
                                 f2_unpack(e2[i][c], e[0], e[1]);
