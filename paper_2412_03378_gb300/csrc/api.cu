@@ -71,7 +71,7 @@ struct vg_workspace {
     bool replay_known = false;            // treplay holds the last forward's replay lengths
     bool tomo_rec = false;                // rec and count are those of the last tomography call with lists, of
     int tomo_n = 0, tomo_a = 0, tomo_w = 0, tomo_h = 0;   // so many Gaussians, angles and detector pixels (one batch)
-    DBuf<uint32_t> treplay, tord_bwd;     // per-tile replay lengths and their order
+    DBuf<uint32_t> treplay, tord_bwd[2];  // per-tile replay lengths and their order, for vg_render_bwd and _noalloc each
     int ppt_fwd = 2, ppt_bwd = 1;         // pixels per thread of the blend kernels
     int tuned_fwd = 0, tuned_bwd = 0;     // vg_autotune's choice (0: none yet)
     int tuned_chunk_fwd = 0, tuned_chunk_bwd = 0;
@@ -293,7 +293,7 @@ vg_status vg_workspace_destroy(vg_workspace *ws) {
     release(ws->tomo_cs);
     release(ws->tord);
     release(ws->treplay);
-    release(ws->tord_bwd);
+    for (auto &b : ws->tord_bwd) release(b);
     release(ws->vbox);
     release(ws->march_E);
     release(ws->march_part);
@@ -334,11 +334,12 @@ static unsigned long long *total64_ptr(vg_workspace *ws) { return ws->counters.p
 static uint32_t *lookback_err_ptr(vg_workspace *ws) { return (uint32_t *)(ws->counters.p + 7); }
 static uint32_t *tomo_changed_ptr(vg_workspace *ws) { return lookback_err_ptr(ws) + 1; }   // h_total[3] when read
 // The backward's tile order: by the replay lengths the last forward measured (longest first), else the binning's.
-static cudaError_t bwd_order(vg_workspace *ws, cudaStream_t st, const int **order) {
+// vg_render_bwd and vg_render_bwd_noalloc share no accumulator and may run on two streams: each has an order of its own.
+static cudaError_t bwd_order(vg_workspace *ws, cudaStream_t st, int noalloc, const int **order) {
     *order = (const int *)ws->tile_order;
     if (!ws->replay_known) return cudaSuccess;
-    *order = (const int *)ws->tord_bwd.p;
-    return launch_tile_order(nullptr, ws->treplay.p, ws->n_tiles, ws->tord_bwd.p, st, &ws->launches);
+    *order = (const int *)ws->tord_bwd[noalloc].p;
+    return launch_tile_order(nullptr, ws->treplay.p, ws->n_tiles, ws->tord_bwd[noalloc].p, st, &ws->launches);
 }
 
 // Reports (and clears) error bits latched on the device: a look-back timeout, a capacity
@@ -711,7 +712,7 @@ static vg_status render_fwd_impl(vg_workspace *ws, float *rgb, float *T_final, v
         VG_CUDA(ws, cudaMemsetAsync(pc, 0, 2 * sizeof(unsigned long long), st));
     }
     VG_TRY(ensure(ws, ws->treplay, (size_t)std::max<long long>(ws->n_tiles, 1), "tile replay lengths"));
-    VG_TRY(ensure(ws, ws->tord_bwd, (size_t)std::max<long long>(ws->n_tiles, 1), "backward tile order"));
+    for (auto &b : ws->tord_bwd) VG_TRY(ensure(ws, b, (size_t)std::max<long long>(ws->n_tiles, 1), "backward tile order"));
     {
         ProfScope ps(ws, ST_FWD, st);
         if (!ws->treplay_clear) VG_CUDA(ws, cudaMemsetAsync(ws->treplay.p, 0, sizeof(uint32_t) * (size_t)ws->n_tiles, st));
@@ -766,7 +767,7 @@ static vg_status render_bwd_impl(vg_workspace *ws, const float *dL_drgb, const f
                                         st, &ws->launches));
         else {
             const int *order;
-            VG_CUDA(ws, bwd_order(ws, st, &order));
+            VG_CUDA(ws, bwd_order(ws, st, 0, &order));
             VG_CUDA(ws, launch_render_bwd(ws->views.p, ws->tile_view.p, order, ws->n_tiles, ws->ranges.p, ws->inst_item,
                                           ws->rec.p, ws->prect.p, ws->bp, ws->ppt_bwd, ws->T_fin.p, ws->S_fin.p,
                                           ws->nlast.p, dL_drgb, dL_dT, ws->grad.p, pc, lookback_err_ptr(ws), st,
@@ -991,7 +992,7 @@ vg_status vg_render_bwd_noalloc(vg_workspace *ws, const float *dL_drgb, const fl
     {
         ProfScope ps(ws, ST_BWD, st);
         const int *order;
-        VG_CUDA(ws, bwd_order(ws, st, &order));
+        VG_CUDA(ws, bwd_order(ws, st, 1, &order));
         VG_CUDA(ws, launch_render_bwd(ws->views.p, ws->tile_view.p, order, ws->n_tiles,
                                       ws->ranges.p, ws->inst_item, ws->rec.p, ws->prect.p, ws->bp, ws->ppt_bwd,
                                       ws->T_fin.p, ws->S_fin.p, ws->nlast.p, dL_drgb, dL_dT, acc, pc,
