@@ -604,6 +604,8 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
         own = cap == cudaStreamCaptureStatusNone;
     }
     if (own) VG_TRY(ensure(ws, ws->hist_tile, tile_words, "radix sort scratch"));
+    else if (known)   // the depth sort's, which the instance buffers may have outgrown
+        VG_TRY(ensure(ws, ws->hist, radix_scratch_words(ws->capacity, bits_for(ws->n_tiles)), "radix sort scratch"));
     // 1. items by depth key (stable: ties keep index order)
     {
         ProfScope ps(ws, ST_DEPTH, st);
