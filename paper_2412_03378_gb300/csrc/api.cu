@@ -103,9 +103,6 @@ constexpr int kDefaultPixelsFwd = 2;
 constexpr long long kOnePixelTiles = 152 * 16;
 constexpr int kDefaultPixelsBwd = 1;
 constexpr int kDefaultChunk = 128;
-// Bytes of a view's weights that stay in an SM's L1 beside the other warps' data: up to there the backward's
-// item order does not matter (200 x 170 pixels, 136 KB: the sort's 45 us would be a third of the backward).
-constexpr long long kTomoL1Image = 160 * 1024;
 constexpr long long kMarchCtas = 4096;   // ray march: CTAs wanted (27 per SM)
 
 enum Stage { ST_PRE, ST_DEPTH, ST_SCAN, ST_DUP, ST_TILE, ST_RANGES, ST_FWD, ST_BWD, ST_CHAIN, ST_LOSS, ST_TFWD,
@@ -1138,28 +1135,20 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
         const long long items = (long long)nb * N;
         if (items >= 0xFFFFFFFFLL) return fail(ws, VG_ERR_INVALID_ARG, "angles x Gaussians per batch must be < 2^32");
         const long long n_tiles = (long long)nb * tpv;
-        // the backward's item order: by the tile of the footprint's centre (the last key: no footprint), once a
-        // view's weights no longer fit one SM's L1
-        const bool by_home = backward && (long long)beam->det_h * tomo_pitch(beam->det_w) * 4 > kTomoL1Image;
         if (lists) {
             VG_TRY(reserve_items(ws, items));
+            VG_TRY(reserve_sort_scratch(ws, items));
         } else {   // what the gradient uses; the buffers that the read-backs describe stay as they are
             VG_TRY(ensure(ws, ws->rec, (size_t)items * kRecF4, "records"));
             VG_TRY(ensure(ws, ws->count, (size_t)items, "tile counts"));
-            for (int k = 0; k < 2 && by_home; ++k) {
-                VG_TRY(ensure(ws, ws->skey[k], (size_t)items, "sort keys"));
-                VG_TRY(ensure(ws, ws->sval[k], (size_t)items, "sort values"));
-            }
         }
-        VG_TRY(reserve_sort_scratch(ws, items));
-        uint32_t *home = ws->skey[0].p, *order = nullptr;
         if (items > 0) {
             ProfScope ps(ws, ST_PRE, st);
             if (lists) VG_CUDA(ws, cudaMemsetAsync(ws->depth.p, 0xFF, sizeof(uint32_t) * (size_t)items, st));
             VG_CUDA(ws, launch_tomo_preprocess(ws->g, ws->tomo_cs.p + 2 * (size_t)a0, nb, beam->det_w, beam->det_h,
                                                beam->pitch_u, beam->pitch_v, beam->u0, beam->v0, opts->tau_cut,
                                                ws->rec.p, ws->count.p, lists ? ws->rect.p : nullptr,
-                                               by_home ? home : nullptr, check ? tomo_changed_ptr(ws) : nullptr, st,
+                                               check ? tomo_changed_ptr(ws) : nullptr, st,
                                                &ws->launches));
         }
         if (check) {
@@ -1234,11 +1223,7 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
             VG_TRY(ensure(ws, ws->grad, (size_t)items * 8, "gradient accumulators"));
             ws->grad_zero_n = 0;   // the tomography backward leaves its sums in the accumulator
             ProfScope ps(ws, ST_TBWD, st);
-            if (by_home)
-                VG_CUDA(ws, launch_radix_sort(home, nullptr, ws->skey[1].p, ws->sval[1].p, ws->skey[0].p, ws->sval[0].p, items,
-                                              nullptr, bits_for(n_tiles + 1), ws->hist.p, lookback_err_ptr(ws), false, &home, &order, st,
-                                              &ws->launches));
-            VG_CUDA(ws, launch_tomo_bwd(items, N, beam->det_w, beam->det_h, order, ws->count.p, ws->rec.p, weights_b, proj_b,
+            VG_CUDA(ws, launch_tomo_bwd(items, N, beam->det_w, beam->det_h, ws->count.p, ws->rec.p, weights_b, proj_b,
                                         dl_b, target_b, scale, ws->grad.p, st, &ws->launches));
             VG_CUDA(ws, launch_tomo_chain(ws->g, ws->tomo_cs.p, A, (long long)a0 * N, items, beam->pitch_u,
                                           beam->pitch_v, beam->u0, beam->v0, ws->grad.p, dmu, dscale, dquat, dkappa,

@@ -82,10 +82,9 @@ template <typename RT>
 __global__ void __launch_bounds__(256)
 k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det_w, int det_h, float pu, float pv,
                   float u0, float v0, float tau_cut, float4 *__restrict__ rec, uint32_t *__restrict__ count,
-                  short4 *__restrict__ rect, uint32_t *__restrict__ home, uint32_t *__restrict__ changed) {
+                  short4 *__restrict__ rect, uint32_t *__restrict__ changed) {
     pdl_entry();
     const long long n_items = (long long)g.n * n_angles;
-    const int tiles_x = (det_w + kTile - 1) / kTile, tiles_y = (det_h + kTile - 1) / kTile;
     for (long long it = (long long)blockIdx.x * blockDim.x + threadIdx.x; it < n_items;
          it += (long long)gridDim.x * blockDim.x) {
         const int a = (int)(it / g.n);
@@ -96,7 +95,7 @@ k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det
         const Density dn = density_of(g, kin, s);
         const float kap = dn.kap;
         short4 rc = make_short4(-1, -1, -1, -1);
-        uint32_t cnt = 0, hm = (uint32_t)n_angles * (uint32_t)(tiles_x * tiles_y);
+        uint32_t cnt = 0;
         if (key_cov(mu, s, q, dn.kap_key, Sig, Rq, qn, smax) && key_k2(dn.kap_key, smax, tau_cut, k2)) {
             // key function: orthographic bounding box of the Mahalanobis-k ellipsoid (FP32, fixed order)
             const float um = VG_ADD(VG_MUL(-st, mu[0]), VG_MUL(ct, mu[1]));
@@ -116,8 +115,6 @@ k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det
             if (ix0 <= ix1 && iy0 <= iy1) {
                 rc = make_short4((short)(ix0 / kTile), (short)(iy0 / kTile), (short)(ix1 / kTile), (short)(iy1 / kTile));
                 cnt = (uint32_t)(rc.z - rc.x + 1) * (uint32_t)(rc.w - rc.y + 1);
-                hm = (uint32_t)a * (uint32_t)(tiles_x * tiles_y) +
-                     (uint32_t)((iy0 + iy1) / (2 * kTile)) * (uint32_t)tiles_x + (uint32_t)((ix0 + ix1) / (2 * kTile));
                 TomoGeom G;
                 tomo_geom(mu, s, Rq, ct, st, pu, pv, u0, v0, G);
                 const float lnA2 = log2f(kap) + kLog2Sqrt2Pi - log2f(G.n);
@@ -133,13 +130,12 @@ k_tomo_preprocess(GaussIn g, const float *__restrict__ cs, int n_angles, int det
         if (changed && count[it] != cnt) *changed = 1u;
         count[it] = cnt;
         if (rect) rect[it] = rc;
-        if (home) home[it] = hm;   // the tile of the rectangle's centre
     }
 }
 
 cudaError_t launch_tomo_preprocess(const GaussIn &g, const float *cs_d, int n_angles, int det_w, int det_h,
                                    float pitch_u, float pitch_v, float u0, float v0, float tau_cut, float4 *rec,
-                                   uint32_t *count, short4 *rect, uint32_t *home, uint32_t *changed, cudaStream_t st,
+                                   uint32_t *count, short4 *rect, uint32_t *changed, cudaStream_t st,
                                    long long *launches) {
     const long long n_items = (long long)g.n * n_angles;
     long long b = (n_items + 255) / 256;
@@ -148,13 +144,13 @@ cudaError_t launch_tomo_preprocess(const GaussIn &g, const float *cs_d, int n_an
     *launches += 1;
     if (g.rec_dtype == VG_BF16)
         pdl_launch(k_tomo_preprocess<__nv_bfloat16>, (unsigned)b, 256, 0, st, g, cs_d, n_angles, det_w, det_h, pitch_u, pitch_v,
-                                                                      u0, v0, tau_cut, rec, count, rect, home, changed);
+                                                                      u0, v0, tau_cut, rec, count, rect, changed);
     else if (g.rec_dtype == VG_F16)
         pdl_launch(k_tomo_preprocess<__half>, (unsigned)b, 256, 0, st, g, cs_d, n_angles, det_w, det_h, pitch_u, pitch_v, u0,
-                                                               v0, tau_cut, rec, count, rect, home, changed);
+                                                               v0, tau_cut, rec, count, rect, changed);
     else
         pdl_launch(k_tomo_preprocess<float>, (unsigned)b, 256, 0, st, g, cs_d, n_angles, det_w, det_h, pitch_u, pitch_v, u0,
-                                                              v0, tau_cut, rec, count, rect, home, changed);
+                                                              v0, tau_cut, rec, count, rect, changed);
     return cudaGetLastError();
 }
 
@@ -344,21 +340,6 @@ cudaError_t launch_tomo_weights(const float *proj, const float *dL, const float 
     return cudaGetLastError();
 }
 
-// One warp per (angle, Gaussian) item: the sum over its pixels needs neither the tile lists nor their
-// order, so a warp walks the item's own pixel rectangle and writes its six sums once -- no
-// reduction per (tile, Gaussian), no atomics, and no pixels of half-covered tiles.  With G = dL/dln tau =
-// weight tau the partials of ln tau = ln A - |y|^2 / 2 follow from sum G, G y and G y y^T in the
-// whitened coordinates, where they are well conditioned for any elongation.  A lane owns eight pixel
-// columns (two 16-byte loads per row, requested a row ahead; columns left or right of the rectangle sit
-// at y0 = kFar, where tau is 0; only an item whose sums come out not finite is summed again with their weights masked,
-// which costs 1.6% here against 7% for masking every row) and every LY-th row, so that a row's shared terms and sums serve
-// eight pixels; 1, 2 or 4 lanes stand side by side, as the rectangle is wide.  The loop is bound by the
-// FMA pipe (a packed instruction holds it for two cycles): about 65 cycles per row of eight pixels.
-// order (may be NULL: item order) lists the items by the tile of their centre and a CTA takes a run of
-// them, so that its warps read the same part of the weights from L1; a warp's items are requested
-// together (one per lane) before the first is summed.  On the workload above 23.7 ms (item sort and chain
-// included) against 62.4 ms for one reduction per (tile, Gaussian) in tile order; without the home order
-// 27 ms, at 1 / 2 / 8 / 32 items a warp 26.9 / 26.1 / 23.6 / 23.4 ms, at 2 or 4 CTAs per SM 25-29 ms.
 // Where the image of weights cannot be had (a fixed-capacity workspace whose buffer is smaller, no memory) a weight is
 // formed where it is used, by the same operations: one value of proj and one of dL (or target) per pixel and item, unaligned.
 struct TomoDirect {
@@ -371,14 +352,29 @@ struct TomoDirect {
     }
 };
 
+// One warp per (angle, Gaussian) item: the sum over its pixels needs neither the tile lists nor their
+// order, so a warp walks the item's own pixel rectangle and writes its six sums once -- no
+// reduction per (tile, Gaussian), no atomics, and no pixels of half-covered tiles.  With G = dL/dln tau =
+// weight tau the partials of ln tau = ln A - |y|^2 / 2 follow from sum G, G y and G y y^T in the
+// whitened coordinates, where they are well conditioned for any elongation.  A lane owns eight pixel
+// columns (two 16-byte loads per row, requested a row ahead; columns left or right of the rectangle sit
+// at y0 = kFar, where tau is 0; only an item whose sums come out not finite is summed again with their weights masked,
+// which costs 1.6% here against 7% for masking every row) and every LY-th row, so that a row's shared terms and sums serve
+// eight pixels; 1, 2 or 4 lanes stand side by side, as the rectangle is wide.  The loop is bound by the
+// FMA pipe (a packed instruction holds it for two cycles): about 65 cycles per row of eight pixels.
+// A warp's items are requested together (one per lane) before the first is summed.  On the workload above 23.7 ms (chain
+// included) against 62.4 ms for one reduction per (tile, Gaussian) in tile order; at 1 / 2 / 4 / 8 / 32 items a warp 30.8 /
+// 27.3 / 25.3 / 24.2 / 23.7 ms, at 2 or 4 CTAs per SM 25-29 ms.  Taking the items by the place of their footprints, so
+// that a CTA's warps share rows of the weights, is worth nothing at 16 items a warp: 23.7 ms there, and with its sort
+// 3% slower at 256 x 256 (1.19 -> 1.22 ms, 50,000 Gaussians), 17% at 200 x 200 (133 -> 156 us, 8,000).
 constexpr int kTomoBwdWarps = 8, kTomoBwdCtas = 3;   // warps per CTA, CTAs per SM
 constexpr int kTomoBwdItems = 16;                    // items of a warp, at most
 
 template <bool DIRECT>   // pitch: floats from row to row of the weights, or of proj and dL
 __global__ void __launch_bounds__(32 * kTomoBwdWarps, kTomoBwdCtas)
-k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch, const uint32_t *__restrict__ order,
-           const uint32_t *__restrict__ count, const float4 *__restrict__ rec, const float *__restrict__ weights,
-           TomoDirect direct, float *__restrict__ acc) {
+k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch, const uint32_t *__restrict__ count,
+           const float4 *__restrict__ rec, const float *__restrict__ weights, TomoDirect direct,
+           float *__restrict__ acc) {
     pdl_entry();
     const int lane = threadIdx.x & 31;
     const long long at0 = (long long)blockIdx.x * kTomoBwdWarps * per_warp + (threadIdx.x >> 5);
@@ -386,8 +382,7 @@ k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch
     float4 my0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f), my1 = my0;
     unsigned my_count = 0;
     if (lane < per_warp && at0 + lane * kTomoBwdWarps < n_items) {
-        const long long at = at0 + lane * kTomoBwdWarps;
-        my_it = order ? (long long)order[at] : at;
+        my_it = at0 + lane * kTomoBwdWarps;
         my_count = count[my_it];
         if (my_count) {
             my0 = __ldg(rec + 2 * my_it);
@@ -490,9 +485,9 @@ k_tomo_bwd(long long n_items, int per_warp, int n_per_view, int det_h, int pitch
     }
 }
 
-cudaError_t launch_tomo_bwd(long long n_items, int n_per_view, int det_w, int det_h, const uint32_t *order,
-                            const uint32_t *count, const float4 *rec, const float *weights, const float *proj,
-                            const float *dL, const float *target, float scale, float *acc, cudaStream_t st,
+cudaError_t launch_tomo_bwd(long long n_items, int n_per_view, int det_w, int det_h, const uint32_t *count,
+                            const float4 *rec, const float *weights, const float *proj, const float *dL,
+                            const float *target, float scale, float *acc, cudaStream_t st,
                             long long *launches) {
     if (n_items <= 0) return cudaSuccess;
     // several items a warp while that leaves four CTAs for every resident one
@@ -502,10 +497,10 @@ cudaError_t launch_tomo_bwd(long long n_items, int n_per_view, int det_w, int de
     const TomoDirect direct{proj, dL, target, scale};
     if (weights)
         pdl_launch(k_tomo_bwd<false>, (unsigned)b, 32 * kTomoBwdWarps, 0, st, n_items, per, n_per_view, det_h, tomo_pitch(det_w),
-                   order, count, rec, weights, direct, acc);
+                   count, rec, weights, direct, acc);
     else
-        pdl_launch(k_tomo_bwd<true>, (unsigned)b, 32 * kTomoBwdWarps, 0, st, n_items, per, n_per_view, det_h, det_w, order, count,
-                   rec, weights, direct, acc);
+        pdl_launch(k_tomo_bwd<true>, (unsigned)b, 32 * kTomoBwdWarps, 0, st, n_items, per, n_per_view, det_h, det_w, count, rec,
+                   weights, direct, acc);
     *launches += 1;
     return cudaGetLastError();
 }

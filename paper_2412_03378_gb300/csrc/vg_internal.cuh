@@ -158,8 +158,8 @@ cudaError_t launch_preprocess(const GaussIn &g, const ViewInfo *views_d, int n_v
 
 cudaError_t launch_tomo_preprocess(const GaussIn &g, const float *cs_d /* [A][2] cos, sin */, int n_angles,
                                    int det_w, int det_h, float pitch_u, float pitch_v, float u0, float v0,
-                                   float tau_cut, float4 *rec, uint32_t *count, short4 *rect, uint32_t *home,
-                                   uint32_t *changed, cudaStream_t st, long long *launches);
+                                   float tau_cut, float4 *rec, uint32_t *count, short4 *rect, uint32_t *changed,
+                                   cudaStream_t st, long long *launches);
 
 // Buffers (16-byte aligned, in 32-bit words) zeroed by one launch.
 struct ClearList {
@@ -297,12 +297,11 @@ cudaError_t launch_tomo_weights(const float *proj, const float *dL, const float 
                                 int n_views, int det_w, int det_h, float *weights, cudaStream_t st,
                                 long long *launches);
 
-// Writes the 8 sums of every item (zeros for one without a footprint) into acc, the items taken in
-// the given order (NULL: their own).  weights NULL: formed from proj and dL (or target and scale) where they are used.
-cudaError_t launch_tomo_bwd(long long n_items, int n_per_view, int det_w, int det_h, const uint32_t *order,
-                            const uint32_t *count, const float4 *rec, const float *weights, const float *proj,
-                            const float *dL, const float *target, float scale, float *acc, cudaStream_t st,
-                            long long *launches);
+// Writes the 8 sums of every item (zeros for one without a footprint) into acc.  weights NULL: formed from proj and dL
+// (or target and scale) where they are used.
+cudaError_t launch_tomo_bwd(long long n_items, int n_per_view, int det_w, int det_h, const uint32_t *count,
+                            const float4 *rec, const float *weights, const float *proj, const float *dL,
+                            const float *target, float scale, float *acc, cudaStream_t st, long long *launches);
 
 cudaError_t launch_tomo_chain(const GaussIn &g, const float *cs_d, int n_angles, long long item0, long long n_items,
                               float pitch_u, float pitch_v, float u0, float v0, const float *grad_acc, float *dmu,
