@@ -106,8 +106,8 @@ typedef struct {
     float z_near;
     uint32_t flags;      /* VG_FLAG_* */
     int32_t pixels_per_thread;  /* blend kernels: pixels owned by one thread, 1, 2 or 4;
-                                   0 = the library defaults (forward 2, backward 1, the
-                                   fastest measured).  Every pixel is evaluated by the same
+                                   0 = the library defaults (forward 1 up to 2,432 tiles and 2
+                                   beyond, backward 1).  Every pixel is evaluated by the same
                                    operations in every layout: images and per-pixel state are
                                    bit-identical, forward and backward take the same skip and
                                    clamp decisions, and gradients differ only in the order of
@@ -349,8 +349,9 @@ vg_status vg_tomo_l2_step(vg_workspace *ws, const vg_gaussians *g, const vg_beam
  * X-ray source is the camera centre and the detector its image plane, so detector pixel (i, j)
  * measures proj = exp(-sum_g tau_g) along that pixel's ray.  Same Gaussians (density only: sh
  * is ignored), the same key function, tile lists and pixel footprint rectangles as vg_preprocess
- * / vg_bin_sort, and the blend kernels in their exact form (no skip, clamp, early stop or
- * background), whose final transmittance is exp(-sum tau).  opts: tau_cut, z_near, flags
+ * / vg_bin_sort; the forward sums tau alone (no skip, clamp, early stop or background) and the
+ * backward walks each item's own rectangle (the blend's backward where pairs are counted, or where
+ * its pixel weights' buffer is missing and may not be allocated).  opts: tau_cut, z_near, flags
  * (VG_FLAG_DENSITY_THETA, VG_FLAG_GRAD_ZERO, VG_FLAG_FIXED_CAPACITY, VG_FLAG_COUNT_PAIRS) and
  * pixels_per_thread are used.  proj [sum_v H_v W_v] float32, device; with dL_dproj non-NULL
  * the gradients of sum(dL_dproj * proj) are accumulated into dmu/dscale/dquat/dkappa as in

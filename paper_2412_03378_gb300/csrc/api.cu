@@ -94,16 +94,24 @@ struct vg_workspace {
 
 namespace {
 
-// Measured on the 1M-Gaussian 1280x832 workload (GB300, footprint culling on): forward
-// 0.53 / 0.49 / 0.74 ms and backward 1.32 / 1.16 / 1.19 ms for 1 / 2 / 4 pixels per thread.
+// Pixels per thread where neither the options nor vg_autotune say.  1 / 2 / 4 of them (backward with its tile order), by tiles:
+//   1,040 (100,000 Gaussians)      forward  94 / 135 / 188 us   backward 160 / 172 / 298 us
+//   1,900 (300,000)                        132 / 161 / 232               212 / 214 / 349
+//   4,160 (1M, 1280 x 832)                 285 / 236 / 354               397 / 386 / 559
+//   5,209 (300,000 in four views, 16 bit)  385 / 420 / 665               508 / 508 / 906
+//   8,160 (1.5M, 1920 x 1080)              489 / 333 / 416               711 / 607 / 775
+// The forward's line follows below; the backward keeps one, although two pay on large images (vg_autotune takes them there).
 constexpr int kDefaultPixelsFwd = 2;
 // Up to this many tiles (16 per SM) the forward takes one pixel per thread: more warps per tile, each with fewer
-// records to visit, and several records evaluated at once.  One / two pixels per thread: 64 tiles 42 / 73 us, 672 tiles
-// 72 / 110 us, 1,040 tiles 93 / 126 us, 1,900 tiles 140 / 178 us, 4,160 tiles 156 / 128 us.
+// records to visit, and several records evaluated at once.  Further one / two pixels per thread: 64 tiles 42 / 73 us,
+// 672 tiles (splat mode) 72 / 110 us.
 constexpr long long kOnePixelTiles = 152 * 16;
 constexpr int kDefaultPixelsBwd = 1;
 constexpr int kDefaultChunk = 128;
-constexpr long long kMarchCtas = 4096;   // ray march: CTAs wanted (27 per SM)
+// Ray march: CTAs wanted (27 per SM), at most kMarchGroups for one tile.  152 / 1,024 / 2,048 / 4,096 / 8,192 CTAs: 320 x 208
+// pixels, 256 samples 698 / 321 / 289 / 296 / 296 us; 384 x 256, 320 samples 1,247 / 770 / 680 / 674 / 685 us; 640 x 480
+// (1,200 tiles) 1,405 / 1,404 / 1,403 / 1,409 / 1,426 us.  A cap of 16, 64 or 256 makes no difference there.
+constexpr long long kMarchCtas = 4096, kMarchGroups = 64;
 
 enum Stage { ST_PRE, ST_DEPTH, ST_SCAN, ST_DUP, ST_TILE, ST_RANGES, ST_FWD, ST_BWD, ST_CHAIN, ST_LOSS, ST_TFWD,
              ST_TBWD, ST_VOXEL, ST_MARCH, ST_COUNT };
@@ -851,7 +859,7 @@ vg_status vg_ray_march(vg_workspace *ws, float t_near, float t_far, int32_t n_sa
     int groups = 1;
     if (ws->opts.T_stop == 0.0f && ws->n_tiles > 0 && ws->n_pixels > 0) {
         const long long px = ws->n_pixels;
-        groups = (int)std::min<long long>(64, (kMarchCtas + ws->n_tiles - 1) / ws->n_tiles);
+        groups = (int)std::min<long long>(kMarchGroups, (kMarchCtas + ws->n_tiles - 1) / ws->n_tiles);
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         VG_CUDA(ws, cudaStreamIsCapturing(st, &cap));
         const bool keep = cap != cudaStreamCaptureStatusNone || (ws->march_part.p && (ws->opts.flags & VG_FLAG_FIXED_CAPACITY));

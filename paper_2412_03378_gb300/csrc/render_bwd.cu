@@ -12,7 +12,8 @@
 //   dL/dA = A sum_p ga u u^T,   dL/dC = C sum_p gq u u^T:
 // per Gaussian only the two symmetric 3x3 moment matrices (6 + 6 values), sum dL/dln(kappa) and
 // the three colour partials are summed (the two matrices' entries packed in pairs, as d' and o' x d' are
-// formed: 0.403 -> 0.386 ms on the 1M-Gaussian 1280 x 832 step, bound by issue slots) -- 16 values, added to the per-item accumulator in L2
+// formed: 0.403 -> 0.386 ms on the 1M-Gaussian 1280 x 832 step, bound by issue slots) -- 16 values, added
+// to the per-item accumulator in L2
 // with vector reductions (red.global.add.v4/v2).  When at most kDirectLanes lanes of the warp
 // contribute to a Gaussian, each of them adds its 16 values directly (four v4 reductions);
 // otherwise three shuffle exchange steps leave every lane with 2 values summed over 8 lanes,
@@ -31,7 +32,12 @@ namespace vg {
 
 // Accumulator layout per item: [0..11] sum of (ga, gq) times xx, xy, x, yy, y, 1 (pairs, as the packed
 // operations leave them), [12] sum dL/dln(kappa), [13..15] dL/dcolour.  Splat mode, where ga = 0: [6..11] sum of gq
-// times the same, one by one (packed with the zeros the backward took 552 against 532 us at 1M Gaussians and 1280 x 832, 190 against 184 at 672 tiles).
+// times the same, one by one (packed with the zeros the backward took 552 against 532 us at 1M Gaussians and
+// 1280 x 832, 190 against 184 us at 672 tiles).
+//
+// The sums reach an accumulator in the order in which the warps arrive, which differs from run to run and, typically,
+// with anything that changes a kernel's timing.  The scale gradients of strongly flattened Gaussians amplify it: two
+// runs of one build are 1e-6 to 4e-5 of the norm apart there, builds of equal arithmetic as much or a little more.
 constexpr int kGradUsed = 16;
 static_assert(kGradUsed == kGradN, "the vector reductions cover the whole 16-float accumulator");
 constexpr int kDirectLanes = 12;   // at most this many contributing lanes: direct reductions
