@@ -189,6 +189,16 @@ vg_status ensure(vg_workspace *ws, DBuf<T> &b, size_t n, const char *what) {
         if (s_ != VG_OK) return s_;        \
     } while (0)
 
+// For a buffer that a faster form wants and the call can do without: whether it may be had.
+template <typename T>
+bool try_ensure(vg_workspace *ws, DBuf<T> &b, size_t n) {
+    if (b.p && b.n >= n) return true;
+    const std::string before = ws->err;
+    if (ensure(ws, b, n, "optional scratch") == VG_OK) return true;
+    ws->err = before;
+    return false;
+}
+
 template <typename T>
 void release(DBuf<T> &b) {
     if (b.p) cudaFree(b.p);
@@ -608,8 +618,8 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
         VG_CUDA(ws, cudaStreamIsCapturing(st, &cap));
         own = cap == cudaStreamCaptureStatusNone;
     }
-    if (own) VG_TRY(ensure(ws, ws->hist_tile, tile_words, "radix sort scratch"));
-    else if (known)   // the depth sort's, which the instance buffers may have outgrown
+    own = own && try_ensure(ws, ws->hist_tile, tile_words);
+    if (known && !own)   // the depth sort's, which the instance buffers may have outgrown
         VG_TRY(ensure(ws, ws->hist, radix_scratch_words(ws->capacity, bits_for(ws->n_tiles)), "radix sort scratch"));
     // 1. items by depth key (stable: ties keep index order)
     {
@@ -694,7 +704,7 @@ vg_status vg_bin_sort(vg_workspace *ws, void *stream) {
             // the binning enqueued ahead still uses the buffers about to be replaced
             if (ahead) VG_CUDA(ws, cudaStreamSynchronize(st));
             VG_TRY(reserve_instances(ws, total));
-            VG_TRY(ensure(ws, ws->hist_tile, radix_scratch_words(ws->capacity, 32), "radix sort scratch"));   // for the next call
+            (void)try_ensure(ws, ws->hist_tile, radix_scratch_words(ws->capacity, 32));   // for the next call
             VG_TRY(bin_rest(total, nullptr, false));
         }
         ws->n_inst = total;
@@ -823,7 +833,7 @@ vg_status vg_project_cone(vg_workspace *ws, const vg_gaussians *g, const vg_came
     VG_TRY(vg_bin_sort(ws, stream));
     if (!proj && ws->n_pixels > 0) return fail(ws, VG_ERR_INVALID_ARG, "proj is NULL");
     // The gradient item by item from pixel weights that the forward writes.  Where their buffer is missing and may
-    // not be allocated (fixed capacity, a capturing stream), and when pairs are counted, the blend's backward runs.
+    // not be allocated (fixed capacity, a capturing stream, no memory), and when pairs are counted, the blend's backward runs.
     bool by_item = dL_dproj && !(opts->flags & VG_FLAG_COUNT_PAIRS);
     if (by_item && (!ws->cone_w.p || ws->cone_w.n < (size_t)ws->n_pixels)) {
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -831,7 +841,7 @@ vg_status vg_project_cone(vg_workspace *ws, const vg_gaussians *g, const vg_came
         if (cap != cudaStreamCaptureStatusNone || (ws->cone_w.p && (opts->flags & VG_FLAG_FIXED_CAPACITY)))
             by_item = false;
         else
-            VG_TRY(ensure(ws, ws->cone_w, (size_t)ws->n_pixels, "pixel weights"));
+            by_item = try_ensure(ws, ws->cone_w, (size_t)ws->n_pixels);
     }
     L2Fused ep{};
     if (by_item) ep.dproj = dL_dproj, ep.weights = ws->cone_w.p;
@@ -865,8 +875,8 @@ vg_status vg_ray_march(vg_workspace *ws, float t_near, float t_far, int32_t n_sa
         const bool keep = cap != cudaStreamCaptureStatusNone || (ws->march_part.p && (ws->opts.flags & VG_FLAG_FIXED_CAPACITY));
         if (keep)
             groups = (int)std::min<long long>(groups, (long long)ws->march_part.n / px);
-        else if (groups > 1)
-            VG_TRY(ensure(ws, ws->march_part, (size_t)(groups * px), "ray-march partial results"));
+        else if (groups > 1 && !try_ensure(ws, ws->march_part, (size_t)(groups * px)))
+            groups = 1;
         groups = std::max(groups, 1);
     }
     ProfScope ps(ws, ST_MARCH, st);
@@ -1116,13 +1126,8 @@ static vg_status tomo_impl(vg_workspace *ws, const vg_gaussians *g, const vg_bea
     while ((long long)batch * tpv >= (1LL << 30) && batch > 1) batch /= 2;
     // the pixels' weights of the backward, an image of padded rows; without it (a fixed-capacity workspace whose buffer is
     // smaller, no memory) the backward forms them from proj where it uses them
-    bool weights = false;
-    if (backward) {
-        const size_t words = (size_t)batch * beam->det_h * tomo_pitch(beam->det_w);
-        if (ws->tomo_dl.n >= words || !ws->tomo_dl.p || !(opts->flags & VG_FLAG_FIXED_CAPACITY))
-            weights = ensure(ws, ws->tomo_dl, words, "pixel weights") == VG_OK;
-        if (!weights) ws->err.clear();
-    }
+    const bool weights =
+        backward && try_ensure(ws, ws->tomo_dl, (size_t)batch * beam->det_h * tomo_pitch(beam->det_w));
     std::vector<float> cs(2 * (size_t)A);
     for (int a = 0; a < A; ++a) {
         if (!std::isfinite(beam->angles[a])) return fail(ws, VG_ERR_INVALID_ARG, "non-finite beam angle");
